@@ -104,7 +104,10 @@ struct March3 {
   static constexpr int OUT = 28;       // output columns per warp
   static constexpr int WARPS = 4;      // warps per block
   static constexpr int NT = 32 * WARPS;
-  static constexpr int MIN_RUN = 8;    // fewest planes per warp before the grid is shrunk
+  // fewest planes per warp before the grid is shrunk: a run of n planes takes n + 4 iterations, and
+  // a small grid is bound by the time of one run, not by the work (48^3: 18.5 us with runs of 8,
+  // 11.7 with runs of 2; 128 x 64 x 64: 21.0 and 17.7)
+  static constexpr int MIN_RUN = 2;
 };
 
 // Batched passes over many independent cases (the sweep of uneven collision cases). One

@@ -33,30 +33,40 @@ __device__ __forceinline__ float sh_up(float v) { return __shfl_up_sync(0xffffff
 __device__ __forceinline__ float sh_dn(float v) { return __shfl_down_sync(0xffffffffu, v, 1); }  // x + 1
 __device__ __forceinline__ int sh_up_i(int v) { return __shfl_up_sync(0xffffffffu, v, 1); }
 __device__ __forceinline__ int sh_dn_i(int v) { return __shfl_down_sync(0xffffffffu, v, 1); }
-__device__ __forceinline__ int sh_dn2_i(int v) { return __shfl_down_sync(0xffffffffu, v, 2); }
 __device__ __forceinline__ float m141(float a, float b, float c) { return __fmaf_rn(4.0f, b, __fadd_rn(a, c)); }
 __device__ __forceinline__ float i2f(int32_t v) { return __int2float_rn(v); }
 
-// minmod of two exact fixed-point differences: the one of smaller magnitude when both have the
-// same sign, else 0.
-__device__ __forceinline__ int32_t mm_i(int32_t a, int32_t b) {
-  const int32_t lo = min(a, b), hi = max(a, b);
-  return lo > 0 ? lo : (hi < 0 ? hi : 0);
+// minmod of two differences: the one of smaller magnitude when both have the same sign, else 0
+// (the median of a, b and 0).
+__device__ __forceinline__ float mm_f(float a, float b) { return fmaxf(fminf(a, b), fminf(fmaxf(a, b), 0.0f)); }
+// 1 / sqrt(x) and x / y for x, y zero or far from the denormal range
+__device__ __forceinline__ float rsqrt_ftz(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
 }
-// Upwind MUSCL state at the face between p and p + e (Eqs. 30-34), in 2^-30 units, from the
-// fixed-point phi at p - e, p, p + e, p + 2e: with (L, C, R) = (p - e, p, p + e) when u_f >= 0
-// and (p + 2e, p + e, p) otherwise, C + minmod(C - L, R - C) / 2; the slopes are exact integers.
-__device__ __forceinline__ float upw_i(float uf, int32_t vm, int32_t v0, int32_t v1, int32_t vp) {
-  const bool pos = uf >= 0.0f;
-  const int32_t L = pos ? vm : vp, C = pos ? v0 : v1, R = pos ? v1 : v0;
-  return __fmaf_rn(0.5f, i2f(mm_i(C - L, R - C)), i2f(C));
+__device__ __forceinline__ float div_ftz(float x, float y) {
+  float r;
+  asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(r) : "f"(x), "f"(y));
+  return r;
 }
 
 // One warp's march over a run of planes. Phi is kept as fixed-point integers; every difference
-// of phi (gradient, diffusion, MUSCL slopes) is taken exactly in integers before it is converted,
+// of phi (gradient, diffusion, MUSCL slopes) is taken exactly in integers and converted once,
 // so stencils keep their precision where phi is close to 1 (a float copy of phi near 1 resolves
 // only 6e-8, which in the liquid interior, where |grad phi| is small but phi (1 - phi) is not,
 // steers the normal of the compressive term). Quantities in 2^-30 units carry the suffix _q.
+// The MUSCL slope of a cell along an axis is the minmod of its two differences there, and both faces
+// of the cell use it (Eqs. 30-34: the upwind state of the face between p and p + e is
+// phi(p) + slope(p) / 2 for u_f >= 0 and phi(p + e) - slope(p + e) / 2 otherwise). The differences are
+// the converted ones that the gradient and the diffusion hold already: rounding to FP32 is monotone
+// and odd, so their minmod is the conversion of the integer minmod. One slope and two states per
+// cell and axis, instead of one integer slope per face, took 256 x 128 x 128 from 71.9 to 68.5 us
+// and 384^3 from 825 to 790 us.
+// It is bound by instruction issue and by dependent operations with two warps per scheduler (255
+// registers). Measured and not kept: rows shared by the warps of a block through shared memory (no
+// warp recomputes its neighbours' rows of a; the halo warps, the barrier per plane and the spills
+// below 168 registers cost more: 81 - 145 us), two rows per thread at 168 registers (74 us).
 // Resident blocks per SM the registers are sized for.
 #ifndef LBM_MARCH_MINB
 #define LBM_MARCH_MINB 2
@@ -95,7 +105,8 @@ __device__ __forceinline__ void march_run(const KParams &P, const int32_t *__res
   const int tx0 = xs / 32, tx1 = min(xs + March3::OUT - 1, nx - 1) / 32;
   unsigned tflag = 0;  // bit 0: tile tx0, bit 1: tile tx1, for the current group of 4 planes
 
-  int32_t I0[NR], I1[NR], NX[NR], Im[M];  // phi of planes p-2, p-1, next (p), and p-3 rows 0..M-1
+  int32_t I0[NR], I1[NR], NX[NR];         // phi of planes p-2, p-1, next (p)
+  float DZk[M], PZk[M];                   // phi(z) - phi(z+1) and the high-side MUSCL state of plane p-2
   float DX0[NR], DX1[NR];                 // phi(x) - phi(x+1) of planes p-2, p-1
   float DY0[NY], DY1[NY];                 // phi(y) - phi(y+1) of planes p-2, p-1
   float XYk[M], YZk[M + 1];               // s_y s_z (phi(x) - phi(x+1)), s_z (phi(y) - phi(y+1)), plane p-2
@@ -109,7 +120,7 @@ __device__ __forceinline__ void march_run(const KParams &P, const int32_t *__res
 #pragma unroll
   for (int i = 0; i < NA; i++) HX0[i] = HX1[i] = HY0[i] = HY1[i] = 0.f;
 #pragma unroll
-  for (int r = 0; r < M; r++) { Im[r] = 0; XYk[r] = 0.f; ASk[r] = 0.f; UZk[r] = 0.f; TZk[r] = 0; }
+  for (int r = 0; r < M; r++) { DZk[r] = PZk[r] = 0.f; XYk[r] = 0.f; ASk[r] = 0.f; UZk[r] = 0.f; TZk[r] = 0; }
 #pragma unroll
   for (int j = 0; j <= M; j++) YZk[j] = 0.f;
 
@@ -146,7 +157,11 @@ __device__ __forceinline__ void march_run(const KParams &P, const int32_t *__res
 #pragma unroll
     for (int j = 0; j < NY; j++) DYp[j] = i2f(I2[j] - I2[j + 1]);
 
-    float XYZ[NA], YZ[NY], ax[NA], ay[NA], ASn[M];
+    float DZn[M];
+#pragma unroll
+    for (int r = 0; r < M; r++) DZn[r] = i2f(I1[r + 2] - I2[r + 2]);
+
+    float XYZ[NA], YZ[NY], ax[NA], ay[NA], ASn[M], PZn[M], MZn[M];
     if (p >= z0) {
       // a = phi (1 - phi) n at plane p - 1, rows -1..M; G = 72 grad(phi) in 2^-30 units
       float XZ[NR];
@@ -164,13 +179,19 @@ __device__ __forceinline__ void march_run(const KParams &P, const int32_t *__res
         const float gy = m141(sh_up(cy), cy, sh_dn(cy));
         const float sz = m141(i2f(I2[i] - I0[i]), i2f(I2[i + 1] - I0[i + 1]), i2f(I2[i + 2] - I0[i + 2]));
         const float gz = m141(sh_up(sz), sz, sh_dn(sz));
-        const float ph = __fmul_rn(i2f(I1[i + 1]), kInvQ30);
+        const float fi = i2f(I1[i + 1]);
+        const float ph = __fmul_rn(fi, kInvQ30);
         const float gg = __fmaf_rn(gx, gx, __fmaf_rn(gy, gy, __fmul_rn(gz, gz)));
-        const float gn = gg > 0.0f ? __fmul_rn(gg, rsqrtf(gg)) : 0.0f;
-        const float sc = __fdividef(__fmul_rn(ph, __fsub_rn(1.0f, ph)), __fadd_rn(gn, e72_q));
+        const float gn = gg > 0.0f ? __fmul_rn(gg, rsqrt_ftz(gg)) : 0.0f;
+        const float sc = div_ftz(__fmul_rn(ph, __fsub_rn(1.0f, ph)), __fadd_rn(gn, e72_q));
         ax[i] = __fmul_rn(gx, sc);
         ay[i] = __fmul_rn(gy, sc);
         az[i] = __fmul_rn(gz, sc);
+        if (i >= 1 && i <= M) {  // MUSCL states of plane p - 1 towards its z faces
+          const float sl = mm_f(DZk[i - 1], DZn[i - 1]);
+          PZn[i - 1] = __fmaf_rn(-0.5f, sl, fi);
+          MZn[i - 1] = __fmaf_rn(0.5f, sl, fi);
+        }
       }
 #pragma unroll
       for (int r = 0; r < M; r++) {
@@ -183,10 +204,9 @@ __device__ __forceinline__ void march_run(const KParams &P, const int32_t *__res
       // z face between planes p-2 and p-1, rows 0..M-1
 #pragma unroll
       for (int r = 0; r < M; r++) {
-        const int32_t v0 = I0[r + 2], v1 = I1[r + 2];
         const float uf = __fmul_rn(0.5f, __fadd_rn(UZk[r], uzn[r]));
-        const float up = upw_i(uf, Im[r], v0, v1, I2[r + 2]);
-        TZn[r] = __float2int_rn(__fmaf_rn(D, i2f(v0 - v1), __fmaf_rn(k3s_q, __fadd_rn(ASk[r], ASn[r]), __fmul_rn(uf, up))));
+        const float up = uf >= 0.0f ? PZk[r] : MZn[r];
+        TZn[r] = __float2int_rn(__fmaf_rn(D, DZk[r], __fmaf_rn(k3s_q, __fadd_rn(ASk[r], ASn[r]), __fmul_rn(uf, up))));
       }
     }
     if (p >= z0 + 2) {
@@ -197,9 +217,11 @@ __device__ __forceinline__ void march_run(const KParams &P, const int32_t *__res
       for (int r = 0; r < M; r++) {
         const float AX = m141(m141(HX0[r], HX1[r], ax[r]), m141(HX0[r + 1], HX1[r + 1], ax[r + 1]),
                               m141(HX0[r + 2], HX1[r + 2], ax[r + 2]));
-        const int32_t v0 = I0[r + 2];
         const float uf = __fmul_rn(0.5f, __fadd_rn(uxk[r], sh_dn(uxk[r])));
-        const float up = upw_i(uf, sh_up_i(v0), v0, sh_dn_i(v0), sh_dn2_i(v0));
+        const float fi = i2f(I0[r + 2]);
+        const float sl = mm_f(sh_up(DX0[r + 2]), DX0[r + 2]);
+        const float px = __fmaf_rn(-0.5f, sl, fi), mx = sh_dn(__fmaf_rn(0.5f, sl, fi));
+        const float up = uf >= 0.0f ? px : mx;
         TX[r] = __float2int_rn(__fmaf_rn(Dx, XYk[r], __fmaf_rn(k3s_q, __fadd_rn(AX, sh_dn(AX)), __fmul_rn(uf, up))));
       }
       float AY[NA];
@@ -208,10 +230,18 @@ __device__ __forceinline__ void march_run(const KParams &P, const int32_t *__res
         const float a = m141(HY0[i], HY1[i], ay[i]);
         AY[i] = m141(sh_up(a), a, sh_dn(a));
       }
+      float PY[NA], MY[NA];  // MUSCL states of rows -1 .. M towards their y faces
+#pragma unroll
+      for (int i = 0; i < NA; i++) {
+        const float fi = i2f(I0[i + 1]);
+        const float sl = mm_f(DY0[i], DY0[i + 1]);
+        PY[i] = __fmaf_rn(-0.5f, sl, fi);
+        MY[i] = __fmaf_rn(0.5f, sl, fi);
+      }
 #pragma unroll
       for (int j = 0; j < M + 1; j++) {  // face between rows j - 1 and j
         const float uf = __fmul_rn(0.5f, __fadd_rn(uyk[j], uyk[j + 1]));
-        const float up = upw_i(uf, I0[j], I0[j + 1], I0[j + 2], I0[j + 3]);
+        const float up = uf >= 0.0f ? PY[j] : MY[j + 1];
         TY[j] = __float2int_rn(__fmaf_rn(Dy, YZk[j], __fmaf_rn(k3s_q, __fadd_rn(AY[j], AY[j + 1]), __fmul_rn(uf, up))));
       }
       bool g0 = false, g1 = false;
@@ -244,7 +274,7 @@ __device__ __forceinline__ void march_run(const KParams &P, const int32_t *__res
     }
     if (p >= z0) {
 #pragma unroll
-      for (int r = 0; r < M; r++) { ASk[r] = ASn[r]; UZk[r] = uzn[r]; XYk[r] = XYZ[r + 1]; }
+      for (int r = 0; r < M; r++) { ASk[r] = ASn[r]; UZk[r] = uzn[r]; XYk[r] = XYZ[r + 1]; PZk[r] = PZn[r]; }
 #pragma unroll
       for (int j = 0; j <= M; j++) YZk[j] = YZ[j + 1];
 #pragma unroll
@@ -254,7 +284,7 @@ __device__ __forceinline__ void march_run(const KParams &P, const int32_t *__res
       }
     }
 #pragma unroll
-    for (int r = 0; r < M; r++) Im[r] = I0[r + 2];
+    for (int r = 0; r < M; r++) DZk[r] = DZn[r];
 #pragma unroll
     for (int i = 0; i < NR; i++) { I0[i] = I1[i]; I1[i] = I2[i]; DX0[i] = DX1[i]; DX1[i] = DXp[i]; }
 #pragma unroll
