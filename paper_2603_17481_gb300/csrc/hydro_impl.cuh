@@ -461,41 +461,69 @@ k_hydro(const KParams P, const typename Store<S>::T *__restrict__ src, typename 
   if (DIM == 3) u_out[2 * NO + (Off)idx] = u2;
 }
 
-// Paired storage access: two populations of x-adjacent cells (x even) as one 8-byte (FP32) or
-// 4-byte (FP16 / BF16) load or store, converted to FP32 as f (loads take w_i, as Store::ld).
+// An element at a 32-bit byte offset from a base that is the same for the whole warp.
+template <class T> __device__ __forceinline__ const T *at(const T *base, unsigned bytes) {
+  return reinterpret_cast<const T *>(reinterpret_cast<const char *>(base) + bytes);
+}
+template <class T> __device__ __forceinline__ T *at(T *base, unsigned bytes) {
+  return reinterpret_cast<T *>(reinterpret_cast<char *>(base) + bytes);
+}
+
+// Paired storage access: the populations of two x-adjacent cells as one 8-byte (FP32) or 4-byte
+// (FP16 / BF16) load (ld, x even) or as two single loads (ld2, from any two places), and their
+// store, converted to FP32 as f (loads take w_i, as Store::ld).
+// w v, never contracted with the sums that follow (2-byte stores keep the bits of the one-cell kernels)
+__device__ __forceinline__ float2 scaled(float2 v, float w) { return make_float2(__fmul_rn(v.x, w), __fmul_rn(v.y, w)); }
 template <int S> struct Pair;
 template <> struct Pair<0> {
   __device__ static __forceinline__ float2 ld(const float *p, float) { return __ldg(reinterpret_cast<const float2 *>(p)); }
-  __device__ static __forceinline__ void st_w(float *p, float a, float b, float w) {
-    *reinterpret_cast<float2 *>(p) = make_float2(w * a, w * b);
+  __device__ static __forceinline__ float2 ld2(const float *a, const float *b, float) {
+    return make_float2(__ldg(a), __ldg(b));
+  }
+  __device__ static __forceinline__ void st_w(float *p, float2 v, float w) {
+    *reinterpret_cast<float2 *>(p) = __fmul2_rn(make_float2(w, w), v);
   }
 };
 template <> struct Pair<1> {
   __device__ static __forceinline__ float2 ld(const __half *p, float w) {
-    const float2 v = __half22float2(__ldg(reinterpret_cast<const __half2 *>(p)));
-    return make_float2(v.x * w, v.y * w);
+    return scaled(__half22float2(__ldg(reinterpret_cast<const __half2 *>(p))), w);
   }
-  __device__ static __forceinline__ void st_w(__half *p, float a, float b, float) {
-    *reinterpret_cast<__half2 *>(p) = __floats2half2_rn(a, b);
+  __device__ static __forceinline__ float2 ld2(const __half *a, const __half *b, float w) {
+    return scaled(make_float2(__half2float(__ldg(a)), __half2float(__ldg(b))), w);
+  }
+  __device__ static __forceinline__ void st_w(__half *p, float2 v, float) {
+    *reinterpret_cast<__half2 *>(p) = __float22half2_rn(v);
   }
 };
 template <> struct Pair<2> {
   __device__ static __forceinline__ float2 ld(const __nv_bfloat16 *p, float w) {
-    const float2 v = __bfloat1622float2(__ldg(reinterpret_cast<const __nv_bfloat162 *>(p)));
-    return make_float2(v.x * w, v.y * w);
+    return scaled(__bfloat1622float2(__ldg(reinterpret_cast<const __nv_bfloat162 *>(p))), w);
   }
-  __device__ static __forceinline__ void st_w(__nv_bfloat16 *p, float a, float b, float) {
-    *reinterpret_cast<__nv_bfloat162 *>(p) = __floats2bfloat162_rn(a, b);
+  __device__ static __forceinline__ float2 ld2(const __nv_bfloat16 *a, const __nv_bfloat16 *b, float w) {
+    return scaled(make_float2(__bfloat162float(__ldg(a)), __bfloat162float(__ldg(b))), w);
+  }
+  __device__ static __forceinline__ void st_w(__nv_bfloat16 *p, float2 v, float) {
+    *reinterpret_cast<__nv_bfloat162 *>(p) = __float22bfloat162_rn(v);
   }
 };
 
-// The 3D hydrodynamic step with two x-adjacent cells per thread (nx even, Q N <= 2^32): a warp
-// covers 64 cells of a row, the block 64 x 4 x 2. For each direction one paired load brings the
-// populations of the source cells x - c_i, x + 1 - c_i when c_x = 0; when c_x = +-1 the pair is
-// shifted by one cell, so one element comes from the neighbouring lane (warp shuffle) or, at the
-// warp's edge, from a single load. Stores of the post-collision populations and of u are paired.
+// The 3D hydrodynamic step with two x-adjacent cells per thread (nx even, Q N <= 2^32). The blocks
+// are 64 x 2 x 2 cells (128 threads), small on purpose: the kernel alternates waiting for memory
+// and computing, so its bandwidth grows with the number of blocks an SM can interleave (six at 80
+// registers; 256 x 128 x 128 D3Q19 FP32 128.5 us, against 142.7 us with three 64 x 4 x 2 blocks of
+// the same registers and this kernel's first form of the loads).
+// For each direction one paired load brings the populations of the source cells x - c_i,
+// x + 1 - c_i when c_x = 0. When c_x = +-1 the pair is shifted by one cell and comes as two single
+// loads: the second one hits the lines of the first in L1, and the thread needs neither its
+// neighbours' registers nor a special case at the edge of the warp (a paired load, a warp shuffle
+// and a load at the warp's edge took 5 instructions and a third register per direction). The base
+// of a direction is the same for all threads and the offsets into it are 32-bit and shared by the
+// directions of a row, so most loads and every store need no address arithmetic of their own.
+// Stores of the post-collision populations and of u are paired.
 // phi of the block + 1 halo is staged in shared memory with the cell x - 1 of lane 0 at an even
-// index, so the four columns x - 1 .. x + 2 of a stencil row are two 8-byte shared loads.
+// index, so the four columns x - 1 .. x + 2 of a stencil row are two 8-byte shared loads. The
+// stencils are evaluated before the pull, which keeps their 36 inputs out of the registers that the
+// populations need.
 // Shared memory of one tile of the paired kernel (the tile is 64 x TY x TZ cells).
 template <int TY, int TZ> struct Hydro2Smem {
   static constexpr int HX = 68, HY = TY + 2, HZ = TZ + 2;  // row pitch 68: column x0 - 1 + j at index j
@@ -505,7 +533,7 @@ template <int TY, int TZ> struct Hydro2Smem {
 // One tile (bx, by, bz) of 64 x TY x TZ cells with a block of 32 x TY x TZ threads. Every thread
 // of the block calls it (one barrier inside; a caller looping over tiles adds one between tiles).
 // halves: bit 0 updates the cells x0 .. x0 + 31 (lanes 0 - 15), bit 1 x0 + 32 .. x0 + 63; the
-// lanes of a half that is not updated still pull (their neighbours' shifted pairs need them).
+// lanes of a half that is not updated only help to stage phi.
 template <class L, int S, int MODE, int TY, int TZ>
 __device__ __forceinline__ void hydro2_tile(const KParams &P, const typename Store<S>::T *__restrict__ src,
                                             typename Store<S>::T *__restrict__ dst, const int32_t *__restrict__ phi,
@@ -522,51 +550,7 @@ __device__ __forceinline__ void hydro2_tile(const KParams &P, const typename Sto
   const int lane = threadIdx.x, ty = threadIdx.y, tz = threadIdx.z;
   const int nx = P.nx, ny = P.ny, nz = P.nz;
   const int x0 = bx * 64, y0 = by * TY, z0 = bz * TZ;
-
   const int x = x0 + 2 * lane, y = y0 + ty, z = z0 + tz;
-  const bool in = x < nx && y < ny && z < nz;  // nx even: x + 1 < nx too
-  const int N = (int)P.N;
-  // row offsets RB[cy + 1][cz + 1] of the neighbourhood and the wrapped columns at the warp's edges
-  int RB[3][3];
-  {
-    const int Y[3] = {y == 0 ? ny - 1 : y - 1, y, y == ny - 1 ? 0 : y + 1};
-    const int Z[3] = {z == 0 ? nz - 1 : z - 1, z, z == nz - 1 ? 0 : z + 1};
-#pragma unroll
-    for (int a = 0; a < 3; a++)
-#pragma unroll
-      for (int b = 0; b < 3; b++) RB[a][b] = nx * (wrapn(Y[a], ny) + ny * Z[b]);
-  }
-  const int xl = x == 0 ? nx - 1 : x - 1;                  // column of x - 1
-  const int xr = x + 2 >= nx ? x + 2 - nx : x + 2;          // column of x + 2
-  const bool edge_l = lane == 0, edge_r = lane == 31 || x + 2 >= nx;
-  const int idx = x + RB[1][1];
-
-  // pull: f_i(x) = src_i(x - c_i), f_i(x + 1) = src_i(x + 1 - c_i), and the fixed-point phi of both
-  // cells (the interfacial gate of the near-contact force)
-  V2 f[L::Q];
-  int2 vg = make_int2(0, 0);
-  auto pull = [&] {
-#pragma unroll
-    for (int i = 0; i < L::Q; i++) {
-      const int cx = L::c(i, 0);
-      const unsigned row = (unsigned)i * (unsigned)N + (unsigned)RB[1 - L::c(i, 1)][1 - L::c(i, 2)];
-      float2 v = make_float2(0.f, 0.f);
-      if (in) v = Pair<S>::ld(src + row + x, L::w(i));
-      if (cx == 0) {
-        f[i].v = v;
-      } else if (cx == 1) {  // sources x - 1, x
-        const float left = __shfl_up_sync(0xffffffffu, v.y, 1);
-        f[i] = V(edge_l ? (in ? Store<S>::ld(src + row + xl, L::w(i)) : 0.f) : left, v.x);
-      } else {  // sources x + 1, x + 2
-        const float right = __shfl_down_sync(0xffffffffu, v.x, 1);
-        f[i] = V(v.y, edge_r ? (in ? Store<S>::ld(src + row + xr, L::w(i)) : 0.f) : right);
-      }
-    }
-    if (in && P.nci_on) vg = *reinterpret_cast<const int2 *>(phi + idx);
-  };
-  // With 2-byte populations the loads are issued before the phi staging and its barrier, so the two
-  // round trips overlap; with FP32 populations (38 values live across the barrier) after it.
-  if constexpr (S != 0) pull();
   // stage phi: the pairs (x0 - 2 + 2 lane, x0 - 1 + 2 lane) of each row cover x0 - 2 .. x0 + 61;
   // lanes 0 and 1 add the pairs at x0 + 62 and x0 + 64 (nx even keeps every pair aligned)
   {
@@ -589,8 +573,8 @@ __device__ __forceinline__ void hydro2_tile(const KParams &P, const typename Sto
     }
   }
   __syncthreads();
-  if constexpr (S == 0) pull();
-  if (!in || !((halves >> (lane >> 4)) & 1u)) return;  // no barrier or shuffle follows
+  // nx even: x + 1 < nx too; no barrier or shuffle follows
+  if (x >= nx || y >= ny || z >= nz || !((halves >> (lane >> 4)) & 1u)) return;
 
   // isotropic gradient and Laplacian of phi (Eqs. 22-23) at both cells: columns x - 1 .. x + 2 of
   // the nine stencil rows as two 8-byte shared loads each
@@ -631,31 +615,61 @@ __device__ __forceinline__ void hydro2_tile(const KParams &P, const typename Sto
   ga0 = __fmul_rn(ga0, 3.0f); ga1 = __fmul_rn(ga1, 3.0f); ga2 = __fmul_rn(ga2, 3.0f); la = __fmul_rn(la, 6.0f);
   gb0 = __fmul_rn(gb0, 3.0f); gb1 = __fmul_rn(gb1, 3.0f); gb2 = __fmul_rn(gb2, 3.0f); lb = __fmul_rn(lb, 6.0f);
 
+  // pull: f_i(x) = src_i(x - c_i), f_i(x + 1) = src_i(x + 1 - c_i). The offsets of the nine source
+  // rows are 32-bit (N <= 2^32 / Q), the base of each direction is common to the warp.
+  using T = typename Store<S>::T;
+  const unsigned N = (unsigned)P.N;
+  unsigned rb[3][3];
+  {
+    const int Y[3] = {y == 0 ? ny - 1 : y - 1, y, y == ny - 1 ? 0 : y + 1};
+    const int Z[3] = {z == 0 ? nz - 1 : z - 1, z, z == nz - 1 ? 0 : z + 1};
+#pragma unroll
+    for (int a = 0; a < 3; a++)
+#pragma unroll
+      for (int b = 0; b < 3; b++) rb[a][b] = (unsigned)(nx * (Y[a] + ny * Z[b]) + x) * (unsigned)sizeof(T);
+  }
+  // from cell x to the cells x - 1 and x + 2, periodic
+  const unsigned dl = (unsigned)((x == 0 ? nx - 1 : -1) * (int)sizeof(T));
+  const unsigned dr = (unsigned)((x + 2 >= nx ? 2 - nx : 2) * (int)sizeof(T));
+  V2 f[L::Q];
+#pragma unroll
+  for (int i = 0; i < L::Q; i++) {
+    const int cx = L::c(i, 0);
+    const unsigned o = rb[1 - L::c(i, 1)][1 - L::c(i, 2)];
+    const T *b = src + (size_t)i * N;
+    if (cx == 0) f[i].v = Pair<S>::ld(at(b, o), L::w(i));
+    else if (cx == 1) f[i].v = Pair<S>::ld2(at(b, o + dl), at(b, o), L::w(i));
+    else f[i].v = Pair<S>::ld2(at(b, o) + 1, at(b, o + dr), L::w(i));
+  }
+  const unsigned idx = rb[1][1] / (unsigned)sizeof(T);
+
+  // the near-contact force where the near-contact kernel wrote one (the gate on the fixed-point phi)
   float4 fra = make_float4(0.f, 0.f, 0.f, 0.f), frb = fra;
   if (P.nci_on) {
+    const int2 vg = *reinterpret_cast<const int2 *>(phi + idx);
     if (q_gate_value(vg.x) >= P.q_th) fra = __ldg(frep + idx);
     if (q_gate_value(vg.y) >= P.q_th) frb = __ldg(frep + idx + 1);
   }
   V2 uo0, uo1, uo2, pso;
   auto store = [&](int i, V2 vw) {
-    if constexpr (MODE == kStep) Pair<S>::st_w(dst + (unsigned)i * (unsigned)N + idx, vw.v.x, vw.v.y, L::w(i));
+    if constexpr (MODE == kStep) Pair<S>::st_w(at(dst + (size_t)i * N, rb[1][1]), vw.v, L::w(i));
   };
   hydro_cell_pair<L, MODE>(P, f, V(pha, phb), V(ga0, gb0), V(ga1, gb1), V(ga2, gb2), V(la, lb), V(fra.x, frb.x),
                            V(fra.y, frb.y), V(fra.z, frb.z), uo0, uo1, uo2, pso, store);
   *reinterpret_cast<float2 *>(u_out + idx) = uo0.v;
-  *reinterpret_cast<float2 *>(u_out + (unsigned)N + idx) = uo1.v;
-  *reinterpret_cast<float2 *>(u_out + 2u * (unsigned)N + idx) = uo2.v;
+  *reinterpret_cast<float2 *>(u_out + (size_t)N + idx) = uo1.v;
+  *reinterpret_cast<float2 *>(u_out + (size_t)N * 2 + idx) = uo2.v;
   if constexpr (MODE == kMoments) *reinterpret_cast<float2 *>(ps_out + idx) = pso.v;
 }
 
 // The near-contact tiles (32 x 8 x 4) holding the two halves of the paired tile (bx, by, bz) of
-// 64 x 4 x 2 cells: tiles 2 bx and 2 bx + 1 of the row (by / 2, bz / 2); the second is -1 beyond
+// 64 x 2 x 2 cells: tiles 2 bx and 2 bx + 1 of the row (by / 4, bz / 2); the second is -1 beyond
 // the grid.
 static_assert(NciTile<3>::X == 32 && NciTile<3>::Y == 8 && NciTile<3>::Z == 4,
-              "a near-contact tile holds 2 x 2 paired tiles of 64 x 4 x 2 cells in y, z, and half of one in x");
+              "a near-contact tile holds 4 x 2 paired tiles of 64 x 2 x 2 cells in y, z, and half of one in x");
 __device__ __forceinline__ int2 nci_tiles_of_pair(const KParams &P, int bx, int by, int bz) {
   const int gtx = (P.nx + 31) >> 5, gty = (P.ny + 7) >> 3;
-  const int t0 = 2 * bx + gtx * ((by >> 1) + gty * (bz >> 1));
+  const int t0 = 2 * bx + gtx * ((by >> 2) + gty * (bz >> 1));
   return make_int2(t0, 2 * bx + 1 < gtx ? t0 + 1 : -1);
 }
 
@@ -687,52 +701,78 @@ __device__ __forceinline__ void hydro2_prefetch(const KParams &P, const typename
   if (PER_LINE < 64 && x0 + PER_LINE < P.nx) asm volatile("prefetch.global.L2 [%0];" ::"l"(row + PER_LINE));
 }
 
+// Tile of the paired kernel in y and z, and the blocks per SM its registers are sized for: D3Q19 six
+// (80 registers; seven at 72 spill and take 130.6 us against 127.0 in FP32, 110.8 against 114.0 in
+// FP16), D3Q27 five (96 registers, 70.7 us on 160 x 96 x 96 against 77.5 with four at 126).
+struct HydroTile {
+  static constexpr int Y = 2, Z = 2;
+};
+template <class L, int S> __host__ __device__ constexpr int hydro2_minb() { return L::Q >= 27 ? 5 : (S == 0 ? 6 : 7); }
+// The blocks that ask L2 for their rows: about the first resident wave of a 152-SM GB300.
+constexpr unsigned kPrefetchBlocks = 912;
+
 // listed == nullptr: every cell. Otherwise the split step's first part: only the halves whose
-// near-contact tile is not listed (a block with both halves listed returns at once). prefetch: the
-// block asks L2 for its population rows before it waits for the previous kernel (D3Q19: 0.9 % off
-// the FP32 step and 1.3 % off the FP16 one on 256 x 128 x 128; D3Q27 measured 2.3 % slower with it,
-// and a prefetch of the tile one resident wave ahead 16 % slower).
+// near-contact tile is not listed (a block with both halves listed returns at once).
+// The first blocks of the grid, which may be resident while the previous kernel still runs, ask L2
+// for their population rows before they wait for it (128.5 -> 127.0 us on 256 x 128 x 128; asked by
+// every block it cost 384^3 6 %: 1785 us against 1682).
 template <class L, int S, int MODE>
-__global__ void __launch_bounds__(256, L::Q >= 27 ? 2 : LBM_HYDRO2_MINB)
+__global__ void __launch_bounds__(32 * HydroTile::Y * HydroTile::Z, hydro2_minb<L, S>())
 k_hydro2(const KParams P, const typename Store<S>::T *__restrict__ src, typename Store<S>::T *__restrict__ dst,
          const int32_t *__restrict__ phi, const float4 *__restrict__ frep, float *__restrict__ u_out,
-         float *__restrict__ ps_out, const int *__restrict__ listed, const bool prefetch) {
+         float *__restrict__ ps_out, const int *__restrict__ listed, const int by0) {
+  constexpr int TY = HydroTile::Y, TZ = HydroTile::Z;
   // the rows were written by an earlier step's hydrodynamic kernel, which has completed; a prefetch
   // only moves lines into L2, the coherence point of every SM
-  if (prefetch) hydro2_prefetch<L, S, 4, 2>(P, src, blockIdx.x, blockIdx.y, blockIdx.z);
+  const int bx = blockIdx.x, by = by0 + blockIdx.y, bz = blockIdx.z;
+  if (blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z) < kPrefetchBlocks)
+    hydro2_prefetch<L, S, TY, TZ>(P, src, bx, by, bz);
   pdl_enter();
   unsigned halves = 3u;
   if (listed) {
-    const int2 t = nci_tiles_of_pair(P, blockIdx.x, blockIdx.y, blockIdx.z);
+    const int2 t = nci_tiles_of_pair(P, bx, by, bz);
     halves = (listed[t.x] ? 0u : 1u) | (t.y >= 0 && listed[t.y] ? 0u : 2u);
     if (halves == 0u) return;  // block-uniform
   }
-  hydro2_tile<L, S, MODE, 4, 2>(P, src, dst, phi, frep, u_out, ps_out, blockIdx.x, blockIdx.y, blockIdx.z, halves);
+  hydro2_tile<L, S, MODE, TY, TZ>(P, src, dst, phi, frep, u_out, ps_out, bx, by, bz, halves);
 }
 
-// The split step's second part: the cells of the listed near-contact tiles. Item i of 4 n covers
-// the paired tile (tx / 2, 2 ty + (i & 1), 2 tz + (i >> 1 & 1)) of listed tile i / 4 = (tx, ty, tz);
+// The split step's second part: the cells of the listed near-contact tiles. Item i of 8 n covers
+// the paired tile (tx / 2, 4 ty + (i & 3), 2 tz + (i >> 2 & 1)) of listed tile i / 8 = (tx, ty, tz);
 // when both near-contact tiles of a pair are listed, the even one's items update both halves and
 // the odd one's items are skipped, so every cell is written once.
 template <class L, int S>
-__global__ void __launch_bounds__(256, L::Q >= 27 ? 2 : LBM_HYDRO2_MINB)
+__global__ void __launch_bounds__(32 * HydroTile::Y * HydroTile::Z, hydro2_minb<L, S>())
 k_hydro2_listed(const KParams P, const typename Store<S>::T *__restrict__ src, typename Store<S>::T *__restrict__ dst,
                 const int32_t *__restrict__ phi, const float4 *__restrict__ frep, float *__restrict__ u_out,
                 const int *__restrict__ tiles, const int *__restrict__ ntiles, const int *__restrict__ listed) {
   pdl_enter();
-  const int n4 = 4 * *ntiles;
+  const int n8 = 8 * *ntiles;
   const int gtx = (P.nx + 31) >> 5, gty = (P.ny + 7) >> 3;
-  for (int it = blockIdx.x; it < n4; it += gridDim.x) {
-    const int tile = tiles[it >> 2];
+  for (int it = blockIdx.x; it < n8; it += gridDim.x) {
+    const int tile = tiles[it >> 3];
     const int tx = tile % gtx, tyz = tile / gtx;
     const int ty = tyz % gty, tz = tyz / gty;
     if ((tx & 1) && listed[tile - 1]) continue;  // block-uniform: the even tile's items cover it
-    const int bx = tx >> 1, by = 2 * ty + (it & 1), bz = 2 * tz + ((it >> 1) & 1);
-    if (4 * by >= P.ny || 2 * bz >= P.nz) continue;
+    const int bx = tx >> 1, by = 4 * ty + (it & 3), bz = 2 * tz + ((it >> 2) & 1);
+    if (HydroTile::Y * by >= P.ny || HydroTile::Z * bz >= P.nz) continue;
     const unsigned halves = (tx & 1) ? 2u : (1u | (tx + 1 < gtx && listed[tile + 1] ? 2u : 0u));
-    hydro2_tile<L, S, kStep, 4, 2>(P, src, dst, phi, frep, u_out, nullptr, bx, by, bz, halves);
+    hydro2_tile<L, S, kStep, HydroTile::Y, HydroTile::Z>(P, src, dst, phi, frep, u_out, nullptr, bx, by, bz, halves);
     __syncthreads();  // the staged phi of this item is no longer read
   }
+}
+
+// k_hydro2 over the whole grid (in several launches where y has more blocks than a grid may).
+template <class L, int S, int MODE>
+cudaError_t launch_hydro2(const KParams &P, const typename Store<S>::T *src, typename Store<S>::T *dst,
+                          const int32_t *phi, const float4 *frep, float *u, float *pstar, const int *listed,
+                          cudaStream_t s) {
+  const int gy = (P.ny + HydroTile::Y - 1) / HydroTile::Y, gz = (P.nz + HydroTile::Z - 1) / HydroTile::Z;
+  cudaError_t e = cudaSuccess;
+  for (int by0 = 0; by0 < gy && e == cudaSuccess; by0 += 65535)
+    e = launch_pdl(k_hydro2<L, S, MODE>, dim3((P.nx + 63) / 64, gy - by0 < 65535 ? gy - by0 : 65535, gz),
+                   dim3(32, HydroTile::Y, HydroTile::Z), 0, s, P, src, dst, phi, frep, u, pstar, listed, by0);
+  return e;
 }
 
 template <class L, int S>
@@ -745,14 +785,10 @@ cudaError_t launch_hydro_t(int mode, const KParams &P, const void *src, void *ds
   const bool i32 = (long long)L::Q * P.N <= (1LL << 32);  // largest offset Q N - 1 fits an unsigned
   const T *a = (const T *)src;
   T *b = (T *)dst;
-  const int *all = nullptr;
   if constexpr (L::D == 3 && S != kStoreRecord) {
     if (i32 && P.nx % 2 == 0) {
-      dim3 g2((P.nx + 63) / 64, (P.ny + 3) / 4, (P.nz + 1) / 2);
-      constexpr bool pf = L::Q == 19;
-      return mode == kStep
-                 ? launch_pdl(k_hydro2<L, S, kStep>, g2, block, 0, s, P, a, b, phi, frep, u, pstar, all, pf)
-                 : launch_pdl(k_hydro2<L, S, kMoments>, g2, block, 0, s, P, a, b, phi, frep, u, pstar, all, false);
+      return mode == kStep ? launch_hydro2<L, S, kStep>(P, a, b, phi, frep, u, pstar, nullptr, s)
+                           : launch_hydro2<L, S, kMoments>(P, a, b, phi, frep, u, pstar, nullptr, s);
     }
   }
   if (mode == kStep)
@@ -782,13 +818,10 @@ cudaError_t launch_split_t(int part, const KParams &P, const void *src, void *ds
   using T = typename Store<S>::T;
   const T *a = (const T *)src;
   T *b = (T *)dst;
-  if (part == 0) {
-    dim3 g2((P.nx + 63) / 64, (P.ny + 3) / 4, (P.nz + 1) / 2);
-    return launch_pdl(k_hydro2<L, S, kStep>, g2, dim3(32, 4, 2), 0, s, P, a, b, phi, frep, u, (float *)nullptr,
-                      (const int *)listed.mark, L::Q == 19);
-  }
-  return launch_pdl(k_hydro2_listed<L, S>, dim3(blocks > 0 ? blocks : 1), dim3(32, 4, 2), 0, s, P, a, b, phi, frep,
-                    u, (const int *)listed.tiles, (const int *)listed.count, (const int *)listed.mark);
+  if (part == 0) return launch_hydro2<L, S, kStep>(P, a, b, phi, frep, u, nullptr, listed.mark, s);
+  return launch_pdl(k_hydro2_listed<L, S>, dim3(blocks > 0 ? 2 * blocks : 1), dim3(32, HydroTile::Y, HydroTile::Z), 0, s,
+                    P, a, b, phi, frep, u, (const int *)listed.tiles, (const int *)listed.count,
+                    (const int *)listed.mark);
 }
 
 template <class L>

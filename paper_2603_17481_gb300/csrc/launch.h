@@ -64,7 +64,7 @@ cudaError_t phase_prepare(int dim);
 cudaError_t launch_hydro(int Q, int store, int mode, const KParams &P, const void *src, void *dst,
                          const int32_t *phi, const float4 *frep, float *u, float *pstar, cudaStream_t s);
 
-// Resident k_hydro2 blocks per SM its registers are sized for (D3Q19; D3Q27 takes 2).
+// Resident k_hydro2_batch blocks (256 threads) per SM its registers are sized for (D3Q19; D3Q27 takes 2).
 #ifndef LBM_HYDRO2_MINB
 #define LBM_HYDRO2_MINB 3
 #endif
@@ -78,9 +78,9 @@ struct TileList {
 };
 
 // The hydrodynamic step split in two launches around the near-contact pass (3D, nx even,
-// Q N <= 2^32: the paired kernel). part 0 updates every 64 x 4 x 2 tile half whose near-contact
+// Q N <= 2^32: the paired kernel). part 0 updates every 64 x 2 x 2 tile half whose near-contact
 // tile is not marked in `listed` (those cells are not gated, so they never read frep, and it may
-// run while the near-contact pass writes frep); part 1 walks the listed tiles on `blocks`
+// run while the near-contact pass writes frep); part 1 walks the listed tiles on 2 `blocks`
 // resident blocks and updates the rest, after the near-contact pass. Each cell is written by
 // exactly one part, with the arithmetic of launch_hydro.
 bool hydro_split_applies(int Q, const KParams &P);
