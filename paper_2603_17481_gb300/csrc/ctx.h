@@ -15,7 +15,6 @@ struct ProfPair {
 struct lbm_ctx {
   lbm_params P;
   lbm::KParams K;
-  lbm::NciTable T;
   long long N;
   size_t pop_bytes;
   cudaStream_t stream = nullptr;
@@ -31,9 +30,9 @@ struct lbm_ctx {
   int32_t *partner = nullptr;
   int *tiles[2] = {nullptr, nullptr};
   int *ntiles = nullptr;  // 2 counters, one per phi buffer
-  int *lflag = nullptr;   // 2 x ntile marks: tile listed for phi[k] (3D)
+  int *lflag = nullptr;   // 2 x ntile marks: tile listed for phi[k]
   int ntile = 0;          // near-contact tiles of the grid
-  lbm::NciAux aux;        // near-contact prefilter buffers (3D grids with sides multiple of 4)
+  lbm::NciAux aux;        // near-contact masks, brick ranges and scan lists
   int nci_blocks = 0;
   // the split step: the near-contact pass and the hydrodynamic update of the listed tiles on the
   // high-priority stream `side`, concurrent with the hydrodynamic update of the other tiles
@@ -70,14 +69,12 @@ inline lbm::TileList tile_list(const lbm_ctx *c, int k) {
   return t;
 }
 
-// The prefilter buffers of the near-contact pass over listed tiles, or nullptr where it does not apply.
-inline const lbm::NciAux *nci_aux(const lbm_ctx *c) { return c->aux.bricks ? &c->aux : nullptr; }
 // Kernels of one near-contact pass over the listed tiles: normals, prefilter (where it applies), scan.
-inline int nci_list_kernels(const lbm_ctx *c) { return nci_aux(c) ? 3 : 2; }
+inline int nci_list_kernels(const lbm_ctx *c) { return lbm::nci_prefilter_applies(c->P.dim, c->K) ? 3 : 2; }
 
 // Enqueues one step of c on stream s from buffers (cur, pcur) (lbm_api.cu); lists = false leaves the
-// near-contact lists as they are. Returns an lbm_status.
-int enqueue_step(lbm_ctx *c, int cur, int pcur, bool lists, cudaStream_t s);
+// near-contact lists as they are; nci_parts as max_parts of launch_nci. Returns an lbm_status.
+int enqueue_step(lbm_ctx *c, int cur, int pcur, bool lists, cudaStream_t s, int nci_parts = lbm::kNciParts);
 
 // Looks up (once per device, current device) the static scratch of lbm_mass_noalloc, which loads
 // its module; lbm_create calls it. Returns an lbm_status.

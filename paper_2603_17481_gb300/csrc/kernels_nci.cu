@@ -5,71 +5,134 @@
 // of the previous step (or over every tile for the diagnostic read-back):
 //   k_nci_normals3 / k_nci_normals2  the normal n = grad(phi) / (|grad(phi)| + eps_n) of every gated
 //                  cell (Eq. 57, isotropic gradient of Eq. 22), computed once and stored as a float4;
-//                  in 3D also zero force at every gated cell and the normal ranges of each 4x4x4 brick;
+//                  zero force at every gated cell (listed tiles); for every row of 32 cells six
+//                  (2D: four) 32-bit masks of its gated cells by the direction of their normals; in
+//                  3D also the normal ranges of each 4x4x4 brick;
 //   k_nci_prefilter (3D, sides multiples of 4) per listed tile, a lower bound of n(x).n(y) from the
-//                  brick ranges; only tiles where the facing gate can hold go on to the scan;
-//   k_nci_scan     per tile: phi and the gated normals of the tile + 3 halo staged in shared memory,
-//                  the gated cells of the tile compacted into a list, then one warp per gated cell
-//                  tests 32 window offsets per iteration in (|r|^2, canonical index) order and
-//                  stops after the first shell holding an accepted candidate.
-// Before scanning, a cell bounds n(x).n(y) from below by the component ranges [lo_a, hi_a] of the
-// gated normals around it: sum_a min(n_a lo_a, n_a hi_a) <= n(x).n(y). A cell whose bound exceeds
-// the facing threshold cannot have a candidate (Eq. 62) and skips the scan; this is exact (a
-// rounding margin of 1e-5 is kept). The ranges are taken first over the whole halo box of the
-// tile, and where that does not decide, over the cell's own 7^3 window: separable sliding min/max
-// filters (z, then y, then x) of the three components, with non-gated cells as NaN (which fminf
-// and fmaxf skip), kept as halves rounded outward (lo down, hi up) so the bound stays a lower
-// bound. A curved interface of radius R turns its normal by about 5/R inside a window, so on
-// isolated drops and bubbles only cells facing another interface within 3 cells are scanned.
+//                  brick ranges; only the half tiles where the facing gate can hold go on to the scan;
+//   k_nci_scan     per unit (half a tile in 3D): the cells that have a possible partner in their
+//                  window by the masks, then one warp per such cell tests its possible partners,
+//                  keeps the nearest accepted one and writes the force. On 3D sides that are not
+//                  multiples of 4 its blocks also make the brick test.
+// The masks are exact: for a cell whose normal's largest component is n_a > 0, a partner with
+// n(x).n(y) <= cos_opp (Eq. 62) has a component m_a below a bound that cos_opp fixes (face_t of the
+// parameters; 0.03 at the paper's -0.8, so partners point the other way along a), and likewise for
+// n_a < 0: class 2 a holds the gated cells with m_a <= face_t, class 2 a + 1 those with m_a >= -face_t.
+// One word answers which cells of a window row may face a cell, so an interface that faces nothing
+// costs 49 words per cell, and the accepted-partner test (Eqs. 59, 61, 62, 65) reads the normals of the
+// few cells that remain.
+// The pass is bound by latency: few units are scanned (20 on 48^3, 60 on 256 x 128 x 128), and a unit is
+// one chain of dependent reads at 700 to 1000 cycles each. So lists are read with their counts,
+// a unit's masks, normals and phi together, and a warp reads several possible partners at once.
+// Staging phi and the normals of a unit + 3 halo in shared memory took 12000 to 15000 cycles alone,
+// and one list of all cells, a warp per cell over all SMs, 7000 to 9000 cycles per cell.
 // The force is written only at gated cells; the hydrodynamic kernel reads it exactly there (same
 // gate function).
 #include "launch.h"
 
 namespace lbm {
 
+// Window radius bound, words of a mask record (one per row of 32 cells) and direction classes.
+constexpr int kWin = 3, kMaskWords = 8;
+template <int DIM> constexpr int kClasses = 2 * DIM;
+
+// The scan's unit of work: half a near-contact tile in 3D (32 x 4 x 4 cells), a tile in 2D.
 template <int DIM> struct NciGeom {
-  static constexpr int TX = NciTile<DIM>::X, TY = NciTile<DIM>::Y, TZ = NciTile<DIM>::Z;
-  static constexpr int H = 3;  // window radius bound
-  static constexpr int HX = TX + 2 * H, HY = TY + 2 * H, HZ = DIM == 3 ? TZ + 2 * H : 1;
-  static constexpr int NB = HX * HY * HZ;
+  static constexpr int TX = NciTile<DIM>::X, TY = DIM == 3 ? NciTile<DIM>::Y / 2 : NciTile<DIM>::Y, TZ = NciTile<DIM>::Z;
+  static constexpr int UNITS = DIM == 3 ? 2 : 1;  // units of a tile, along y
   static constexpr int NT = TX * TY * TZ, NW = NT / 32;
-  static constexpr int NZR = HX * HY * TZ;  // z-filtered planes (3D)
-  static constexpr int NYR = HX * TY * TZ;  // z- and y-filtered rows
-  static constexpr size_t smem = sizeof(int32_t) * NB + sizeof(float) * 3 * NB + sizeof(int) * (NT + 1) +
-                                 sizeof(float) * (6 * (NW + 1) + 1) + sizeof(long long) * (HY * HZ + 1) +
-                                 sizeof(int) * HX + sizeof(__half) * 6 * ((DIM == 3 ? NZR : 0) + NYR) +
-                                 sizeof(float) * NB;
 };
 
-// The eight windows [o, o + 6], o = 0..7, of fourteen values: the suffix extremes of [0, 6] and the
-// prefix extremes of [7, 13] (van Herk / Gil-Werman), 18 operations instead of 48.
-template <bool MAX>
-__device__ __forceinline__ void win7x8(const float *v, float *out) {
-  auto op = [](float a, float b) { return MAX ? fmaxf(a, b) : fminf(a, b); };
-  float suf[7], pre[7];
-  suf[6] = v[6];
-#pragma unroll
-  for (int i = 5; i >= 0; i--) suf[i] = op(v[i], suf[i + 1]);
-  pre[0] = v[7];
-#pragma unroll
-  for (int j = 1; j < 7; j++) pre[j] = op(pre[j - 1], v[7 + j]);
-  out[0] = suf[0];
-#pragma unroll
-  for (int o = 1; o < 7; o++) out[o] = op(suf[o], pre[o - 1]);
-  out[7] = pre[6];
+// The masks of the rows around a unit: 38 columns (bit j of a row: column x0 - 3 + j, in two words),
+// TY + 6 by TZ + 6 rows (2D: one plane).
+template <int DIM> struct MaskBox {
+  using G = NciGeom<DIM>;
+  static constexpr int COLS = 32 + 2 * kWin, HY = G::TY + 2 * kWin, HZ = DIM == 3 ? G::TZ + 2 * kWin : 1, ROWS = HY * HZ;
+  uint2 m[kClasses<DIM>][ROWS];
+};
+
+// The direction class whose members may face a cell with normal n: the axis of its largest component.
+template <int DIM> __device__ __forceinline__ int facing_class(const float4 &n) {
+  const float a0 = fabsf(n.x), a1 = fabsf(n.y), a2 = fabsf(n.z);
+  if (DIM == 3 && a2 > a0 && a2 > a1) return 4 + (n.z > 0.0f ? 0 : 1);
+  if (a1 > a0) return 2 + (n.y > 0.0f ? 0 : 1);
+  return n.x > 0.0f ? 0 : 1;
 }
 
-// The four windows [o, o + 6], o = 0..3, of ten values share the core [3, 6] and the pairs (1, 2)
-// and (7, 8): 13 min (or max) operations instead of 24.
-template <bool MAX>
-__device__ __forceinline__ void win7x4(const float *v, float *out) {
-  auto op = [](float a, float b) { return MAX ? fmaxf(a, b) : fminf(a, b); };
-  const float core = op(op(v[3], v[4]), op(v[5], v[6]));
-  const float p12 = op(v[1], v[2]), q78 = op(v[7], v[8]);
-  out[0] = op(core, op(v[0], p12));
-  out[1] = op(core, op(p12, v[7]));
-  out[2] = op(core, op(v[2], q78));
-  out[3] = op(core, op(q78, v[9]));
+// Writes the mask record of one row of 32 cells (the warp's; g: this lane's cell is gated, n its normal).
+template <int DIM>
+__device__ __forceinline__ void store_masks(const KParams &P, unsigned *__restrict__ rec, bool g, float n0, float n1,
+                                            float n2, int lane) {
+  const float a[3] = {n0, n1, n2};
+  unsigned mine = 0;
+  if (__any_sync(0xffffffffu, g)) {
+#pragma unroll
+    for (int c = 0; c < kClasses<DIM>; c++) {
+      const unsigned m = __ballot_sync(0xffffffffu, g && ((c & 1) ? a[c >> 1] >= -P.face_t : a[c >> 1] <= P.face_t));
+      if (lane == c) mine = m;
+    }
+  }
+  if (lane < kClasses<DIM>) rec[lane] = mine;
+}
+
+// Fills the mask box (all zero on entry) of the unit at (x0, y0, z0), threads tid of nt. A row of 38 columns of
+// the periodic grid is made of pieces that end at a word's or the grid's edge, three where nx is a
+// multiple of 32; each thread takes one piece of a row, so all reads are in flight together. A piece
+// in a tile that is not listed has no gated cell (its record is of an older step); mark == nullptr:
+// every tile is listed.
+template <int DIM>
+__device__ __forceinline__ void stage_masks(const KParams &P, MaskBox<DIM> &box, const unsigned *__restrict__ masks,
+                                            const int *__restrict__ mark, int gtx, int gty, int x0, int y0, int z0,
+                                            int tid, int nt) {
+  using M = MaskBox<DIM>;
+  const int nx = P.nx, s = wrapn(x0 - kWin, nx);
+  // pieces per row: a word's piece is at least 32 columns except at the ends and at the grid's edge
+  const int pieces = nx % 32 == 0 ? 3 : 3 + 2 * (M::COLS / nx + 1);
+  for (int it = tid; it < pieces * M::ROWS; it += nt) {
+    const int r = it % M::ROWS, k = it / M::ROWS;
+    int col = s, pos = 0, take = 0;
+    for (int j = 0;; j++) {
+      take = min(min(32 - (col & 31), nx - col), M::COLS - pos);
+      if (j == k || take == 0) break;
+      pos += take;
+      col += take;
+      if (col == nx) col = 0;
+    }
+    if (take == 0) continue;
+    const int y = wrapn(y0 - kWin + r % M::HY, P.ny), z = DIM == 3 ? wrapn(z0 - kWin + r / M::HY, P.nz) : 0;
+    const uint4 *rec = reinterpret_cast<const uint4 *>(masks) +
+                       kMaskWords / 4 * ((col >> 5) + gtx * (y + (long long)P.ny * z));
+    const uint4 a = rec[0];
+    const uint2 b = DIM == 3 ? *reinterpret_cast<const uint2 *>(rec + 1) : make_uint2(0u, 0u);
+    if (mark && !mark[(col >> 5) + gtx * (y / NciTile<DIM>::Y + gty * (z / NciTile<DIM>::Z))]) continue;
+    const unsigned w[6] = {a.x, a.y, a.z, a.w, b.x, b.y};
+#pragma unroll
+    for (int c = 0; c < kClasses<DIM>; c++) {
+      const unsigned v = take == 32 ? w[c] : (w[c] >> (col & 31)) & ((1u << take) - 1u);
+      if (!v) continue;
+      const unsigned long long p = (unsigned long long)v << pos;
+      if ((unsigned)p) atomicOr(&box.m[c][r].x, (unsigned)p);
+      if (p >> 32) atomicOr(&box.m[c][r].y, (unsigned)(p >> 32));
+    }
+  }
+}
+
+// The possible partners (7 columns x - 3 .. x + 3, bits above are not cleared) of the cell in column cx in
+// a row of its class.
+__device__ __forceinline__ unsigned window_bits(const uint2 &row, int cx) { return __funnelshift_r(row.x, row.y, cx); }
+
+// Whether the cell in column tx, row (ty, tz) of the unit, with normal n, has a possible partner in its
+// window of radius W.
+template <int DIM, int W>
+__device__ __forceinline__ bool may_face(const MaskBox<DIM> &box, const float4 &n, int tx, int ty, int tz) {
+  using M = MaskBox<DIM>;
+  const uint2 *m = box.m[facing_class<DIM>(n)] + (DIM == 3 ? (tz + kWin) * M::HY : 0) + ty + kWin;
+  unsigned any = 0;
+#pragma unroll
+  for (int dz = DIM == 3 ? -W : 0; dz <= (DIM == 3 ? W : 0); dz++)
+#pragma unroll
+    for (int dy = -W; dy <= W; dy++) any |= window_bits(m[dz * M::HY + dy], tx);
+  return (any & (((1u << (2 * W + 1)) - 1u) << (kWin - W))) != 0u;
 }
 
 template <int DIM>
@@ -79,50 +142,58 @@ __device__ __forceinline__ void tile_of(int tile, int gtx, int gty, int &bx, int
   bz = tile / (gtx * gty);
 }
 
-// Normals of the gated cells of the listed tiles (or of every tile when tiles == nullptr), 2D.
+// Normals, masks and zero force of the gated cells of the listed tiles (or normals and masks of every
+// tile when tiles == nullptr), 2D: a warp per row of a tile.
 __global__ void __launch_bounds__(NciGeom<2>::NT)
-k_nci_normals2(const KParams P, const int32_t *__restrict__ phi, float4 *__restrict__ nrm,
+k_nci_normals2(const KParams P, const int32_t *__restrict__ phi, float4 *__restrict__ nrm, float4 *__restrict__ frep,
                const int *__restrict__ tiles, const int *__restrict__ ntiles, int total, int gtx, int gty,
-               int *__restrict__ reset_other) {
+               unsigned *__restrict__ masks, int *__restrict__ reset_other) {
   pdl_enter();
   if (reset_other && blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0) *reset_other = 0;
   using G = NciGeom<2>;
   using SL = StencilOf<2>::type;
+  const int first = tiles ? tiles[blockIdx.x] : 0;  // in flight with the count (the list has room for every tile)
   const int n = tiles ? *ntiles : total;
   const int nx = P.nx, ny = P.ny;
   for (int t = blockIdx.x; t < n; t += gridDim.x) {
     int bx, by, bz;
-    tile_of<2>(tiles ? tiles[t] : t, gtx, gty, bx, by, bz);
+    tile_of<2>(!tiles ? t : (t == (int)blockIdx.x ? first : tiles[t]), gtx, gty, bx, by, bz);
     const int x = bx * G::TX + threadIdx.x, y = by * G::TY + threadIdx.y;
-    if (x >= nx || y >= ny) continue;
-    const int X[3] = {x == 0 ? nx - 1 : x - 1, x, x == nx - 1 ? 0 : x + 1};
-    const int Y[3] = {y == 0 ? ny - 1 : y - 1, y, y == ny - 1 ? 0 : y + 1};
+    if (y >= ny) continue;  // the whole warp
     const long long idx = (long long)x + (long long)nx * y;
-    if (!(q_gate_value(phi[idx]) >= P.q_th)) continue;
+    const bool g = x < nx && q_gate_value(phi[idx]) >= P.q_th;
     float g0 = 0.f, g1 = 0.f;
+    if (g) {
+      const int X[3] = {x == 0 ? nx - 1 : x - 1, x, x == nx - 1 ? 0 : x + 1};
+      const int Y[3] = {y == 0 ? ny - 1 : y - 1, y, y == ny - 1 ? 0 : y + 1};
 #pragma unroll
-    for (int i = 1; i < SL::Q; i++) {
-      if (!positive<SL>(i)) continue;
-      const int c0 = SL::c(i, 0), c1 = SL::c(i, 1);
-      const float d = SL::w(i) * dphi_of(__ldg(phi + X[1 + c0] + (long long)nx * Y[1 + c1]),
-                                         __ldg(phi + X[1 - c0] + (long long)nx * Y[1 - c1]));
-      g0 += c0 * d;
-      g1 += c1 * d;
+      for (int i = 1; i < SL::Q; i++) {
+        if (!positive<SL>(i)) continue;
+        const int c0 = SL::c(i, 0), c1 = SL::c(i, 1);
+        const float d = SL::w(i) * dphi_of(__ldg(phi + X[1 + c0] + (long long)nx * Y[1 + c1]),
+                                           __ldg(phi + X[1 - c0] + (long long)nx * Y[1 - c1]));
+        g0 += c0 * d;
+        g1 += c1 * d;
+      }
+      g0 *= 3.0f; g1 *= 3.0f;
+      const float inv = 1.0f / (sqrtf(g0 * g0 + g1 * g1) + P.eps_n);
+      g0 = g0 * inv; g1 = g1 * inv;
+      nrm[idx] = make_float4(g0, g1, 0.0f, 0.0f);
+      if (tiles) frep[idx] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    g0 *= 3.0f; g1 *= 3.0f;
-    const float inv = 1.0f / (sqrtf(g0 * g0 + g1 * g1) + P.eps_n);
-    nrm[idx] = make_float4(g0 * inv, g1 * inv, 0.0f, 0.0f);
+    store_masks<2>(P, masks + (long long)kMaskWords * (bx + (long long)gtx * y), g, g0, g1, 0.f, threadIdx.x);
   }
 }
 
 // Normals of the gated cells of the listed tiles (or of every tile when tiles == nullptr), 3D.
 // One 128-thread block per half tile (32 x 4 x 4 cells, eight 4x4x4 bricks side by side in x):
 // phi of the half tile + 1 halo (34 x 6 x 6) is staged in shared memory, then warp w takes the 4
-// rows of plane z0 + w. The gradient is the isotropic D3Q27 one of Eq. 22, summed over the 13
-// links in the same order as everywhere else.
-// With the prefilter (listed tiles): every gated cell's force is set to zero here (the scan
-// overwrites it where a partner is found), the tile's flag is set, and the component ranges of
-// the gated normals of each brick are stored (empty bricks as [+inf, -inf]).
+// rows of plane z0 + w (a thread per cell spends more on the bricks than it gains in latency: 414
+// against 164 us on the 384^3 swarm, 13.9 against 7.2 on 256 x 128 x 128). The gradient is the
+// isotropic D3Q27 one of Eq. 22, summed over the 13 links in the same order as everywhere else.
+// On listed tiles every gated cell's force is set to zero here (it is overwritten where a partner is
+// found) and, with the bricks, the component ranges of the gated normals of each brick are stored (empty bricks as [+inf, -inf]; cells beyond the grid in the last brick of a side
+// that is not a multiple of 4 count as not gated).
 constexpr int kNrmThreads = 128;
 struct NrmBox {
   static constexpr int X = 34, Y = 6, Z = 6, ROWS = Y * Z;  // warp w stages rows w, w + 4, ...
@@ -133,26 +204,28 @@ k_nci_normals3(const KParams P, const int32_t *__restrict__ phi, float4 *__restr
                const int *__restrict__ tiles, const int *__restrict__ ntiles, int total, int gtx, int gty,
                const NciAux aux, int *__restrict__ reset_other) {
   pdl_enter();
-  if (reset_other && blockIdx.x == 0 && threadIdx.x == 0) *reset_other = 0;
   using G = NciGeom<3>;
   using SL = StencilOf<3>::type;
   using B = NrmBox;
-  static_assert(G::TX == 32 && G::TY == 8 && G::TZ == 4, "two 32 x 4 x 4 halves per tile");
+  static_assert(G::TX == 32 && G::TY == 4 && G::TZ == 4, "half a near-contact tile");
   __shared__ int32_t s_box[B::ROWS * B::X];
   __shared__ float s_part[4][8][6];  // [warp][brick][lo0..hi2]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const bool bricks = aux.bricks != nullptr;  // uniform over the grid
-  if (bricks && blockIdx.x == 0 && threadIdx.x == 0) *aux.nscan = 0;
+  const int first = tiles ? tiles[blockIdx.x >> 1] : 0;  // in flight with the count (the list has room for every tile)
   const int n = tiles ? *ntiles : total;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (reset_other) *reset_other = 0;
+    if (bricks) *aux.nscan = 0;
+  }
   const int nx = P.nx, ny = P.ny, nz = P.nz;
   const float inf = __int_as_float(0x7f800000);
   for (int item = blockIdx.x; item < 2 * n; item += gridDim.x) {
-    const int tile = tiles ? tiles[item >> 1] : (item >> 1);
+    const int tile = !tiles ? (item >> 1) : (item == (int)blockIdx.x ? first : tiles[item >> 1]);
     const int half = item & 1;
     int bx, by, bz;
     tile_of<3>(tile, gtx, gty, bx, by, bz);
-    if (bricks && half == 0 && threadIdx.x == 0) aux.flags[tile] = 1;
-    const int x0 = bx * G::TX, y0 = by * G::TY + 4 * half, z0 = bz * G::TZ;
+    const int x0 = bx * G::TX, y0 = by * NciTile<3>::Y + 4 * half, z0 = bz * G::TZ;
     {
       const int xa = wrapn(x0 - 1 + lane, nx), xb = wrapn(x0 + 31 + (lane & 1), nx);
       int32_t va[9], vb[9];
@@ -178,28 +251,31 @@ k_nci_normals3(const KParams P, const int32_t *__restrict__ phi, float4 *__restr
     for (int r = 0; r < 4; r++) {
       const int y = y0 + r;
       const int o = ((warp + 1) * B::Y + r + 1) * B::X + lane + 1;
-      if (!(xin && y < ny && q_gate_value(s_box[o]) >= P.q_th)) continue;
+      const bool g = xin && y < ny && q_gate_value(s_box[o]) >= P.q_th;
       float g0 = 0.f, g1 = 0.f, g2 = 0.f;
+      if (g) {
 #pragma unroll
-      for (int i = 1; i < SL::Q; i++) {
-        if (!positive<SL>(i)) continue;
-        const int c0 = SL::c(i, 0), c1 = SL::c(i, 1), c2 = SL::c(i, 2);
-        const int off = c0 + B::X * (c1 + B::Y * c2);
-        const float d = SL::w(i) * dphi_of(s_box[o + off], s_box[o - off]);
-        g0 += c0 * d;
-        g1 += c1 * d;
-        g2 += c2 * d;
-      }
-      g0 *= 3.0f; g1 *= 3.0f; g2 *= 3.0f;
-      const float inv = 1.0f / (sqrtf(g0 * g0 + g1 * g1 + g2 * g2) + P.eps_n);
-      g0 *= inv; g1 *= inv; g2 *= inv;
-      const long long idx = (long long)x + (long long)nx * (y + (long long)ny * z);
-      nrm[idx] = make_float4(g0, g1, g2, 0.0f);
-      if (bricks) {
-        frep[idx] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int i = 1; i < SL::Q; i++) {
+          if (!positive<SL>(i)) continue;
+          const int c0 = SL::c(i, 0), c1 = SL::c(i, 1), c2 = SL::c(i, 2);
+          const int off = c0 + B::X * (c1 + B::Y * c2);
+          const float d = SL::w(i) * dphi_of(s_box[o + off], s_box[o - off]);
+          g0 += c0 * d;
+          g1 += c1 * d;
+          g2 += c2 * d;
+        }
+        g0 *= 3.0f; g1 *= 3.0f; g2 *= 3.0f;
+        const float inv = 1.0f / (sqrtf(g0 * g0 + g1 * g1 + g2 * g2) + P.eps_n);
+        g0 *= inv; g1 *= inv; g2 *= inv;
+        const long long idx = (long long)x + (long long)nx * (y + (long long)ny * z);
+        nrm[idx] = make_float4(g0, g1, g2, 0.0f);
+        if (tiles) frep[idx] = make_float4(0.f, 0.f, 0.f, 0.f);
         lo0 = fminf(lo0, g0); lo1 = fminf(lo1, g1); lo2 = fminf(lo2, g2);
         hi0 = fmaxf(hi0, g0); hi1 = fmaxf(hi1, g1); hi2 = fmaxf(hi2, g2);
       }
+      if (y < ny && z < nz)  // the whole warp
+        store_masks<3>(P, aux.masks + (long long)kMaskWords * (bx + (long long)gtx * (y + (long long)ny * z)), g, g0, g1,
+                       g2, lane);
     }
     if (bricks) {  // lanes 4k..4k+3 of each warp share brick k; the four planes meet in shared memory
 #pragma unroll
@@ -220,7 +296,7 @@ k_nci_normals3(const KParams P, const int32_t *__restrict__ phi, float4 *__restr
     if (bricks) {
       const int k = threadIdx.x;
       const int gbx = 8 * bx + k, gby = 2 * by + half;
-      if (k < 8 && gbx < (nx >> 2) && gby < (ny >> 2)) {
+      if (k < 8 && gbx < ((nx + 3) >> 2) && gby < ((ny + 3) >> 2)) {
         float v[6];
 #pragma unroll
         for (int c = 0; c < 6; c++) {
@@ -234,504 +310,461 @@ k_nci_normals3(const KParams P, const int32_t *__restrict__ phi, float4 *__restr
         o.y = h(__float2half_rd(v[2]));
         o.z = h(__float2half_ru(v[3])) | (h(__float2half_ru(v[4])) << 16);
         o.w = h(__float2half_ru(v[5]));
-        aux.bricks[(long long)gbx + (long long)(nx >> 2) * (gby + (long long)(ny >> 2) * bz)] = o;
+        aux.bricks[(long long)gbx + (long long)((nx + 3) >> 2) * (gby + (long long)((ny + 3) >> 2) * bz)] = o;
       }
     }
   }
 }
 
-// One 128-thread block per listed tile (3D). The tile's sixteen bricks are tested against the
-// union of the normal ranges of their 27 neighbouring bricks, a 10x4x3 box of bricks; a brick of a
-// tile that is not listed holds no gated cell and counts as empty. Every window offset of the scan
-// (each component |r_a| <= 3) stays inside those 27 bricks, so for a cell x of a brick with ranges
-// [lo, hi] and every gated y in its window,
-//   n(x).n(y) >= sum_a min(lo_a L_a, lo_a H_a, hi_a L_a, hi_a H_a),
-// [L, H] being the union (the product is bilinear, so its minimum over the two boxes is at a
-// corner). Where that bound exceeds cos_opp + 1e-5 for all sixteen bricks, no cell of the tile
-// can meet the facing gate (Eq. 62) and the tile keeps the zero force written by the normals
-// pass; otherwise the tile goes to the scan list.
-__global__ void __launch_bounds__(128)
-k_nci_prefilter(const KParams P, const uint4 *__restrict__ bricks, const unsigned char *__restrict__ flags,
-                const int *__restrict__ tiles, const int *__restrict__ ntiles, int *__restrict__ scan_tiles,
-                int *__restrict__ nscan, int gtx, int gty) {
+// Component ranges of the gated normals of some cells: lo0..2, hi0..2.
+struct NrmRange {
+  float v[6];
+};
+
+// The union of the ranges of the bricks that hold the cells 4 jx .. 4 jx + 3 (and likewise in y and z) of
+// the periodic grid; a brick of a tile that is not listed holds no gated cell and counts as empty.
+// Where a side is a multiple of 4 the four cells are one brick; elsewhere they may touch up to three
+// (the last brick of the side is short). At most one axis in four starts a new brick per cell, so
+// the loops below run once per distinct brick. ALIGNED: every side is a multiple of 4.
+template <bool ALIGNED>
+__device__ __forceinline__ NrmRange brick_range(const KParams &P, const uint4 *__restrict__ bricks,
+                                                const int *__restrict__ mark, int gtx, int gty, int jx, int jy, int jz) {
+  const float inf = __int_as_float(0x7f800000);
+  NrmRange r{{inf, inf, inf, -inf, -inf, -inf}};
+  const int nbx = (P.nx + 3) >> 2, nby = (P.ny + 3) >> 2;
+  const bool ax = !ALIGNED && (P.nx & 3), ay = !ALIGNED && (P.ny & 3), az = !ALIGNED && (P.nz & 3);
+  int pz = -1;
+  for (int cz = 0; cz < (az ? 4 : 1); cz++) {
+    const int bz = ALIGNED ? wrapn(jz, P.nz >> 2) : wrapn(4 * jz + cz, P.nz) >> 2;
+    if (bz == pz) continue;
+    pz = bz;
+    int py = -1;
+    for (int cy = 0; cy < (ay ? 4 : 1); cy++) {
+      const int by = ALIGNED ? wrapn(jy, P.ny >> 2) : wrapn(4 * jy + cy, P.ny) >> 2;
+      if (by == py) continue;
+      py = by;
+      int px = -1;
+      for (int cx = 0; cx < (ax ? 4 : 1); cx++) {
+        const int bx = ALIGNED ? wrapn(jx, P.nx >> 2) : wrapn(4 * jx + cx, P.nx) >> 2;
+        if (bx == px) continue;
+        px = bx;
+        const uint4 w = bricks[(long long)bx + (long long)nbx * (by + (long long)nby * bz)];
+        if (!mark[(bx >> 3) + gtx * ((by >> 1) + gty * bz)]) continue;
+        const auto lo = [](unsigned u) { return __half2float(__ushort_as_half((unsigned short)(u & 0xffffu))); };
+        const auto hi = [](unsigned u) { return __half2float(__ushort_as_half((unsigned short)(u >> 16))); };
+        r.v[0] = fminf(r.v[0], lo(w.x)); r.v[1] = fminf(r.v[1], hi(w.x)); r.v[2] = fminf(r.v[2], lo(w.y));
+        r.v[3] = fmaxf(r.v[3], lo(w.z)); r.v[4] = fmaxf(r.v[4], hi(w.z)); r.v[5] = fmaxf(r.v[5], lo(w.w));
+      }
+    }
+  }
+  return r;
+}
+
+// A lower bound of n(x).n(y) over the cells x of the brick whose ranges are entry rc of the staged box
+// (s_r[component][entry], entries RX wide and RY high) and every gated cell y of their windows, along
+// axis a. Every window offset of the scan (each component |r_a| <= 3) stays inside the 27 entries
+// around the brick, so with [L, H] their union
+//   n(x).n(y) >= sum_a min(lo_a L_a, lo_a H_a, hi_a L_a, hi_a H_a)
+// (the product is bilinear, so its minimum over the two boxes is at a corner).
+template <int RX, int RY, int NR>
+__device__ __forceinline__ float brick_bound(const float (*s_r)[NR], int a, int rc) {
+  const float inf = __int_as_float(0x7f800000);
+  float L = inf, H = -inf;
+#pragma unroll
+  for (int dz = -1; dz <= 1; dz++)
+#pragma unroll
+    for (int dy = -1; dy <= 1; dy++)
+#pragma unroll
+      for (int dx = -1; dx <= 1; dx++) {
+        const int r = rc + dx + RX * (dy + RY * dz);
+        L = fminf(L, s_r[a][r]);
+        H = fmaxf(H, s_r[3 + a][r]);
+      }
+  const float lo = s_r[a][rc], hi = s_r[3 + a][rc];
+  return fminf(fminf(lo * L, lo * H), fminf(hi * L, hi * H));
+}
+
+// One 128-thread block per listed tile (3D, sides multiples of 4). The tile's sixteen bricks are
+// tested against the union of the normal ranges of their 27 neighbouring bricks, a 10x4x3 box of
+// bricks. Where the bound exceeds cos_opp + 1e-5 for all eight bricks of a half tile, none of its
+// cells can meet the facing gate (Eq. 62) and the half keeps the zero force written by the normals
+// pass; otherwise it goes to the scan list. mark: the tiles listed for this phi.
+__global__ void __launch_bounds__(128, 12)
+k_nci_prefilter(const KParams P, const NciAux aux, const int *__restrict__ mark, const int *__restrict__ tiles,
+                const int *__restrict__ ntiles, int gtx, int gty) {
   pdl_enter();
   constexpr int RX = 10, RY = 4, RZ = 3, NR = RX * RY * RZ;
   __shared__ float s_r[6][NR];
   __shared__ float s_b[48];
   const int tid = threadIdx.x;
+  const int first = tiles[blockIdx.x];  // in flight with the count (the list has room for every tile)
   const int n = *ntiles;
-  const int nbx = P.nx >> 2, nby = P.ny >> 2, nbz = P.nz >> 2;
-  const float inf = __int_as_float(0x7f800000);
+  const int nbx = P.nx >> 2, nby = P.ny >> 2;
   const float thr = P.cos_opp + 1e-5f;
   for (int t = blockIdx.x; t < n; t += gridDim.x) {
-    const int tile = tiles[t];
+    const int tile = t == (int)blockIdx.x ? first : tiles[t];
     int bx, by, bz;
     tile_of<3>(tile, gtx, gty, bx, by, bz);
     if (tid < NR) {
       const int rx = tid % RX, ry = (tid / RX) % RY, rz = tid / (RX * RY);
-      const int gbx = wrapn(8 * bx - 1 + rx, nbx), gby = wrapn(2 * by - 1 + ry, nby), gbz = wrapn(bz - 1 + rz, nbz);
-      float v[6] = {inf, inf, inf, -inf, -inf, -inf};
-      if (flags[(gbx >> 3) + gtx * ((gby >> 1) + gty * gbz)]) {
-        const uint4 w = bricks[(long long)gbx + (long long)nbx * (gby + (long long)nby * gbz)];
-        v[0] = __half2float(__ushort_as_half((unsigned short)(w.x & 0xffffu)));
-        v[1] = __half2float(__ushort_as_half((unsigned short)(w.x >> 16)));
-        v[2] = __half2float(__ushort_as_half((unsigned short)(w.y & 0xffffu)));
-        v[3] = __half2float(__ushort_as_half((unsigned short)(w.z & 0xffffu)));
-        v[4] = __half2float(__ushort_as_half((unsigned short)(w.z >> 16)));
-        v[5] = __half2float(__ushort_as_half((unsigned short)(w.w & 0xffffu)));
-      }
+      const NrmRange r = brick_range<true>(P, aux.bricks, mark, gtx, gty, 8 * bx - 1 + rx, 2 * by - 1 + ry, bz - 1 + rz);
 #pragma unroll
-      for (int c = 0; c < 6; c++) s_r[c][tid] = v[c];
+      for (int c = 0; c < 6; c++) s_r[c][tid] = r.v[c];
     }
     __syncthreads();
-    if (tid < 48) {
-      const int b = tid & 15, a = tid >> 4;
-      const int cx = b & 7, cy = b >> 3;
-      float L = inf, H = -inf;
-#pragma unroll
-      for (int dz = 0; dz < 3; dz++)
-#pragma unroll
-        for (int dy = 0; dy < 3; dy++)
-#pragma unroll
-          for (int dx = 0; dx < 3; dx++) {
-            const int r = (cx + dx) + RX * ((cy + dy) + RY * dz);
-            L = fminf(L, s_r[a][r]);
-            H = fmaxf(H, s_r[3 + a][r]);
-          }
-      const int rc = (cx + 1) + RX * ((cy + 1) + RY);
-      const float lo = s_r[a][rc], hi = s_r[3 + a][rc];
-      s_b[tid] = fminf(fminf(lo * L, lo * H), fminf(hi * L, hi * H));
-    }
+    const int rc = ((tid & 7) + 1) + RX * (((tid >> 3) & 1) + 1 + RY);
+    if (tid < 48) s_b[tid] = brick_bound<RX, RY, NR>(s_r, tid >> 4, rc);
     __syncthreads();
-    bool need = false;
-    if (tid < 16) {
-      const int cx = tid & 7, cy = tid >> 3;
-      const int rc = (cx + 1) + RX * ((cy + 1) + RY);
-      const bool has = 8 * bx + cx < nbx && 2 * by + cy < nby && s_r[0][rc] <= s_r[3][rc];
-      need = has && s_b[tid] + s_b[16 + tid] + s_b[32 + tid] <= thr;
+    if (tid < 32) {
+      const int b = tid & 15;
+      const bool has = tid < 16 && 8 * bx + (tid & 7) < nbx && 2 * by + (tid >> 3) < nby && s_r[0][rc] <= s_r[3][rc];
+      const unsigned need = __ballot_sync(0xffffffffu, has && s_b[b] + s_b[16 + b] + s_b[32 + b] <= thr);
+      if (tid < 2 && ((need >> (8 * tid)) & 0xffu)) aux.scan_units[atomicAdd(aux.nscan, 1)] = 2 * tile + tid;
     }
-    if (__syncthreads_or(need) && tid == 0) scan_tiles[atomicAdd(nscan, 1)] = tile;
+    __syncthreads();  // s_r and s_b are free for the next tile
   }
 }
 
+// The window of radius W: row r of a cell's window is (dy, dz), entry r * (2 W + 1) + dx + W in canonical order.
+template <int DIM, int W> struct Window {
+  static constexpr int SIDE = 2 * W + 1, ROWS = DIM == 3 ? SIDE * SIDE : SIDE;
+  static constexpr int CELLS = SIDE * ROWS;
+  __device__ static int dy(int r) { return r % SIDE - W; }
+  __device__ static int dz(int r) { return DIM == 3 ? r / SIDE - W : 0; }
+};
+// The cell at a window offset of (x, y, z), periodic.
 template <int DIM>
-__global__ void __launch_bounds__(NciGeom<DIM>::NT, NciGeom<DIM>::NT >= 1024 ? 1 : 2)
-k_nci_scan(const KParams P, const NciTable T, const int32_t *__restrict__ phi, const float4 *__restrict__ nrm,
-           float4 *__restrict__ frep, int32_t *__restrict__ partner, int debug, const int *__restrict__ tiles,
-           const int *__restrict__ ntiles, int total, int gtx, int gty, unsigned char *__restrict__ flags,
-           const int *__restrict__ listed, const int *__restrict__ nlisted) {
-  pdl_enter();
-  using G = NciGeom<DIM>;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  int32_t *s_phi = reinterpret_cast<int32_t *>(smem_raw);
-  float *s_n = reinterpret_cast<float *>(s_phi + G::NB);
-  int *s_list = reinterpret_cast<int *>(s_n + 3 * G::NB);
-  int *s_count = s_list + G::NT;
-  float *s_rng = reinterpret_cast<float *>(s_count + 1);  // [NW + 1][6]
-  long long *s_row = reinterpret_cast<long long *>(s_rng + 6 * (G::NW + 1) + 1);  // [HY * HZ], 8-aligned
-  int *s_col = reinterpret_cast<int *>(s_row + G::HY * G::HZ);                   // [HX]
-  __half *s_yr = reinterpret_cast<__half *>(s_col + G::HX);                        // [6][NYR]
-  __half *s_zr = s_yr + 6 * G::NYR;                                                // [6][NZR] (3D)
-  // q = phi (1 - phi) of the staged box (phi clamped, binary32 as the gate takes it), computed once
-  float *s_q = reinterpret_cast<float *>(s_zr + 6 * (DIM == 3 ? G::NZR : 0));        // [NB]
+__device__ __forceinline__ long long window_cell(const KParams &P, int x, int y, int z, int dx, int dy, int dz) {
+  return (long long)wrapn(x + dx, P.nx) +
+         (long long)P.nx * (wrapn(y + dy, P.ny) + (long long)P.ny * (DIM == 3 ? wrapn(z + dz, P.nz) : 0));
+}
 
+// The partner of one cell (Eqs. 59-65), by a warp: candidate criteria Eqs. 59, 61, 62; the winner is the
+// nearest accepted candidate, then the largest facing score, then the first in the window's canonical
+// order, which the packed key |r|^2 - 31 bits of the score - 9 bits of the entry orders exactly; all
+// ones: none. m: the cell's row of its class (pitch HY in z); list: room for the window's cells. The
+// possible partners are listed first, so that every lane reads as many as the others.
+template <int DIM, int W>
+__device__ __forceinline__ unsigned long long pair_of(const KParams &P, const int32_t *__restrict__ phi,
+                                                      const float4 *__restrict__ nrm, int x, int y, int z,
+                                                      const float4 &me, const int32_t vx, int lane, const uint2 *m, int cx,
+                                                      unsigned short *list) {
+  using Win = Window<DIM, W>;
+  int cand = 0;
+#pragma unroll
+  for (int k = 0; k < (Win::ROWS + 31) / 32; k++) {
+    const int r = lane + 32 * k;
+    unsigned b = 0;
+    if (r < Win::ROWS) {
+      const int dz = Win::dz(r), dy = Win::dy(r);
+      b = (window_bits(m[(DIM == 3 ? dz * MaskBox<DIM>::HY : 0) + dy], cx) >> (kWin - W)) & ((1u << Win::SIDE) - 1u);
+      if (dy == 0 && dz == 0) b &= ~(1u << W);  // the cell itself
+    }
+    // entries of the lanes before this one
+    int at = __popc(b);
+    const int own = at;
+#pragma unroll
+    for (int sh = 1; sh < 32; sh <<= 1) {
+      const int o = __shfl_up_sync(0xffffffffu, at, sh);
+      if (lane >= sh) at += o;
+    }
+    const int all = __shfl_sync(0xffffffffu, at, 31);
+    at += cand - own;
+    cand += all;
+    while (b) {
+      list[at++] = (unsigned short)(r * Win::SIDE + __ffs(b) - 1);
+      b &= b - 1u;
+    }
+  }
+  __syncwarp();
+  const float n0 = me.x, n1 = me.y, n2 = me.z, qxc = q_gate_value(vx);
+  const float sim = __fmul_rn(P.eta, fmaxf(qxc, P.eps_q));
+  unsigned long long best = ~0ull;
+  constexpr int AT = 4;  // read together
+  for (int i0 = lane; i0 < cand; i0 += 32 * AT) {
+    int e[AT];
+    int32_t vy[AT];
+    float4 o[AT];
+#pragma unroll
+    for (int j = 0; j < AT; j++) {
+      const int i = i0 + 32 * j;
+      e[j] = i < cand ? list[i] : -1;
+      if (e[j] >= 0) {
+        const int r = e[j] / Win::SIDE, dx = e[j] % Win::SIDE - W;
+        const long long q = window_cell<DIM>(P, x, y, z, dx, Win::dy(r), Win::dz(r));
+        vy[j] = phi[q];
+        o[j] = __ldg(nrm + q);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < AT; j++) {
+      if (e[j] < 0) continue;
+      const float qy = q_gate_value(vy[j]);
+      if (fabsf(__fsub_rn(qy, qxc)) <= sim) {
+        const float dot = __fadd_rn(__fadd_rn(__fmul_rn(n0, o[j].x), __fmul_rn(n1, o[j].y)), __fmul_rn(n2, o[j].z));
+        if (dot <= P.cos_opp) {
+          const float ff = fmaxf(-dot, 0.0f);
+          const int r = e[j] / Win::SIDE, dx = e[j] % Win::SIDE - W, dy = Win::dy(r), dz = Win::dz(r);
+          const unsigned long long key = ((unsigned long long)(dx * dx + dy * dy + dz * dz) << 40) |
+                                         ((unsigned long long)(0x7fffffffu - __float_as_uint(ff)) << 9) |
+                                         (unsigned long long)e[j];
+          best = key < best ? key : best;
+        }
+      }
+    }
+  }
+  __syncwarp();  // the list is free for the warp's next cell
+  if (__any_sync(0xffffffffu, best != ~0ull)) {
+#pragma unroll
+    for (int sh = 16; sh > 0; sh >>= 1) {
+      const unsigned long long other = __shfl_xor_sync(0xffffffffu, best, sh);
+      best = other < best ? other : best;
+    }
+  }
+  return best;
+}
+
+// The force of a cell on its partner's key (Eqs. 66-73), and the partner where asked for.
+template <int DIM, int W>
+__device__ __forceinline__ void pair_force(const KParams &P, const int32_t *__restrict__ phi,
+                                           const float4 *__restrict__ nrm, float4 *__restrict__ frep,
+                                           int32_t *__restrict__ partner, int x, int y, int z, const float4 &me,
+                                           const int32_t vx, const unsigned long long best) {
+  using Win = Window<DIM, W>;
+  const float n0 = me.x, n1 = me.y, n2 = me.z, qxc = q_gate_value(vx);
+  const long long gidx = window_cell<DIM>(P, x, y, z, 0, 0, 0);
+  const int bj = (int)(best & 511ull), od2 = (int)(best >> 40), r = bj / Win::SIDE;
+  const int dx = bj % Win::SIDE - W, dy = Win::dy(r), dz = Win::dz(r);
+  const float ff = __uint_as_float(0x7fffffffu - (unsigned)((best >> 9) & 0x7fffffffull));
+  const long long gy = window_cell<DIM>(P, x, y, z, dx, dy, dz);
+  const int32_t vy = phi[gy];
+  const float4 o = __ldg(nrm + gy);
+  const float m0 = o.x, m1 = o.y, m2 = o.z;
+  const float qy = q_gate_value(vy);
+  // paired indicator and clamp, Eqs. 66-67
+  const float qpair = 0.5f * (qxc + qy);
+  const float qcl = fminf(fmaxf(qpair, P.eps_q), 0.25f - P.eps_q);
+  // proximity indicator, Eq. 70, as eps * artanh(sqrt(1 - 4 q)): the same value, and
+  // 1 - 4 q_pair = ((1 - 2 phi_x)^2 + (1 - 2 phi_y)^2) / 2 has no cancellation
+  float mm;
+  if (qcl == qpair) {
+    const float ax = 1.0f - 2.0f * fminf(fmaxf(phi_of(vx), 0.f), 1.f);
+    const float ay = 1.0f - 2.0f * fminf(fmaxf(phi_of(vy), 0.f), 1.f);
+    mm = 0.5f * (ax * ax + ay * ay);
+  } else {
+    mm = 1.0f - 4.0f * qcl;
+  }
+  const float h = P.eps * atanhf(sqrtf(mm));
+  const float tt = h / P.h0;
+  const float tp = (P.p == 4.0f) ? (tt * tt) * (tt * tt) : powf(tt, P.p);
+  const float wh = 1.0f / (1.0f + tp);  // Eq. 71
+  // symmetric normal, Eq. 69, line-of-centres fallback, oriented toward the partner
+  const float rn = sqrtf((float)od2);
+  const float r0 = dx / rn, r1 = dy / rn, r2 = dz / rn;
+  float s0 = n0 - m0, s1 = n1 - m1, s2 = n2 - m2;
+  const float sn = sqrtf(s0 * s0 + s1 * s1 + s2 * s2);
+  if (sn < 1e-8f) {
+    s0 = r0; s1 = r1; s2 = r2;
+  } else {
+    const float is = 1.0f / (sn + P.eps_n);
+    s0 *= is; s1 *= is; s2 *= is;
+  }
+  if (r0 * s0 + r1 * s1 + r2 * s2 < 0.0f) {
+    s0 = -s0; s1 = -s1; s2 = -s2;
+  }
+  // flux and force density with the facing factor of Eq. 68, Eqs. 72-73
+  const float rho = P.rho_g + P.drho * phi_of(vx);
+  const float amp = rho * P.A_rep * qcl * wh * ff;
+  frep[gidx] = make_float4(amp * s0, amp * s1, DIM == 3 ? amp * s2 : 0.0f, 1.0f);
+  if (partner) {
+    partner[3 * gidx] = dx;
+    partner[3 * gidx + 1] = dy;
+    partner[3 * gidx + 2] = dz;
+  }
+}
+
+// list: the units to scan (tile * UNITS + half), or with per_tile the tiles whose units to scan, and their
+// count; nullptr: every unit, with zero force and no partner first written at every cell (the
+// read-back). With bricks (3D) each unit is first tested against the ranges of the bricks around it,
+// as in the prefilter. mark: the tiles listed for this phi (nullptr: all).
+template <int DIM, int W>
+__global__ void __launch_bounds__(NciGeom<DIM>::NT, 2)
+k_nci_scan(const KParams P, const int32_t *__restrict__ phi, const float4 *__restrict__ nrm,
+           float4 *__restrict__ frep, int32_t *__restrict__ partner, const int *__restrict__ list,
+           const int *__restrict__ count, bool per_tile, int total, int gtx, int gty, const unsigned *__restrict__ masks,
+           const uint4 *__restrict__ bricks, const int *__restrict__ mark, const int max_parts) {
+  using G = NciGeom<DIM>;
+  using M = MaskBox<DIM>;
+  constexpr int RX = 10, RY = 3, RZ = 3, NR = RX * RY * RZ;
+  __shared__ M s_box;
+  __shared__ float s_r[DIM == 3 ? 6 : 1][NR];
+  __shared__ float s_b[24];
+  __shared__ int s_list[G::NT];
+  __shared__ float4 s_n[G::NT];  // normals of the listed cells
+  __shared__ int32_t s_v[G::NT];  // and their phi
+  __shared__ unsigned long long s_best[G::NT];  // and their partners
+  __shared__ unsigned short s_cand[G::NW][Window<DIM, W>::CELLS];
+  __shared__ int s_count;
   const int tx = threadIdx.x, ty = threadIdx.y, tz = threadIdx.z;
   const int tid = tx + G::TX * (ty + G::TY * tz), lane = tid & 31, warp = tid >> 5;
   const int nx = P.nx, ny = P.ny, nz = P.nz;
-  const int n = tiles ? *ntiles : total;
-  if (flags) {  // the prefilter has read the flags of this step's listed tiles: clear them
-    const int m = *nlisted;
-    for (int i = blockIdx.x * G::NT + tid; i < m; i += gridDim.x * G::NT) flags[listed[i]] = 0;
-  }
+  pdl_enter();
+  const int per = per_tile ? G::UNITS : 1;
+  const int n = list ? *count * per : total;
+  // Where there are fewer units than blocks several blocks take the same one, each a share of its cells
+  // by position (a film's 70 cells are then one round of the block's 16 warps instead of five: 48^3 35.2 ->
+  // 34.0 us a step); the tests before that are repeated by each, in the time one of them takes. max_parts
+  // is 1 where other cases use the SMs meanwhile (a batch: nine film cases 222 us with 8, 211 with 1).
+  int parts = 1;
+  while (parts < max_parts && 2 * parts * n <= (int)gridDim.x) parts *= 2;
 
-  for (int t = blockIdx.x; t < n; t += gridDim.x) {
+  for (int item = blockIdx.x; item < n * parts; item += gridDim.x) {
+    const int t = item / parts, part = item - t * parts;
+    int u = list ? list[t / per] : t;
+    if (per_tile) u = u * G::UNITS + t % G::UNITS;
+    const int half = u % G::UNITS;
     int bx, by, bz;
-    tile_of<DIM>(tiles ? tiles[t] : t, gtx, gty, bx, by, bz);
-    const int x0 = bx * G::TX, y0 = by * G::TY, z0 = bz * G::TZ;
+    tile_of<DIM>(u / G::UNITS, gtx, gty, bx, by, bz);
+    if constexpr (DIM == 3) {
+      if (bricks) {
+        if (tid < NR) {
+          const int rx = tid % RX, ry = (tid / RX) % RY, rz = tid / (RX * RY);
+          const NrmRange r =
+              brick_range<false>(P, bricks, mark, gtx, gty, 8 * bx - 1 + rx, 2 * by + half - 1 + ry, bz - 1 + rz);
+#pragma unroll
+          for (int c = 0; c < 6; c++) s_r[c][tid] = r.v[c];
+        }
+        __syncthreads();
+        const int rc = ((tid & 7) + 1) + RX * (1 + RY);
+        if (tid < 24) s_b[tid] = brick_bound<RX, RY, NR>(s_r, tid >> 3, rc);
+        __syncthreads();
+        const bool has = tid < 8 && 32 * bx + 4 * tid < nx && 8 * by + 4 * half < ny && s_r[0][rc] <= s_r[3][rc];
+        const bool need = has && s_b[tid] + s_b[8 + tid] + s_b[16 + tid] <= P.cos_opp + 1e-5f;
+        if (!__syncthreads_or(need)) continue;  // uniform over the block
+      }
+    }
+    const int x0 = bx * G::TX, y0 = by * NciTile<DIM>::Y + half * G::TY, z0 = bz * G::TZ;
     const int x = x0 + tx, y = y0 + ty, z = z0 + tz;
     const bool inb = x < nx && y < ny && z < nz;
     const long long idx = inb ? (long long)x + (long long)nx * (y + (long long)ny * z) : 0;
-    bool gated = false;
-    if (!tiles) {  // every tile is visited: skip those without an interfacial cell
-      gated = inb && (q_gate_value(phi[idx]) >= P.q_th);
-      if (!__syncthreads_or(gated)) {
-        if (debug && inb) {
-          frep[idx] = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (partner) partner[3 * idx] = partner[3 * idx + 1] = partner[3 * idx + 2] = INT32_MIN;
-        }
-        continue;  // uniform over the block
-      }
-    }
-
-    // Stage phi and the gated normals (written once per step by k_nci_normals) of the tile + 3
-    // halo, row by row (rows of HX = TX + 6 values): every row's phi loads are issued before any is
-    // stored; each warp then gates its own rows and loads the normals of their gated cells.
-    // Non-gated cells hold NaN normals, which fminf / fmaxf skip.
-    float lo0 = 1e30f, lo1 = 1e30f, lo2 = 1e30f, hi0 = -1e30f, hi1 = -1e30f, hi2 = -1e30f;
-    {
-      constexpr int NROWS = G::HY * G::HZ, RPW = (NROWS + G::NW - 1) / G::NW;
-      const int xl = wrapn(x0 - G::H + tx, nx);
-      const int xr = wrapn(x0 - G::H + 32 + (tx & 7), nx);
-      const bool xtra = lane < G::HX - 32;
-      int32_t va[RPW], vb[RPW];
-#pragma unroll
-      for (int h = 0; h < RPW; h++) {
-        const int r = warp + h * G::NW;
-        if (r < NROWS) {
-          const int ry = r % G::HY, rz = r / G::HY;
-          const long long row = (long long)nx * (wrapn(y0 + ry - G::H, ny) +
-                                                 (long long)ny * (DIM == 3 ? wrapn(z0 + rz - G::H, nz) : 0));
-          if (lane == 0) s_row[r] = row;
-          va[h] = phi[row + xl];
-          if (xtra) vb[h] = phi[row + xr];
-        }
-      }
-#pragma unroll
-      for (int h = 0; h < RPW; h++) {
-        const int r = warp + h * G::NW;
-        if (r < NROWS) {
-          s_phi[r * G::HX + lane] = va[h];
-          s_q[r * G::HX + lane] = q_gate_value(va[h]);
-          if (xtra) {
-            s_phi[r * G::HX + 32 + lane] = vb[h];
-            s_q[r * G::HX + 32 + lane] = q_gate_value(vb[h]);
-          }
-        }
-      }
-      __syncwarp();  // this warp's rows of s_phi and s_row
-      const float qnan = __int_as_float(0x7fffffff);
-#pragma unroll 2
-      for (int h = 0; h < RPW; h++) {
-        const int r = warp + h * G::NW;
-        if (r >= NROWS) break;
-        const int b = r * G::HX + lane;
-        const bool ga = s_q[b] >= P.q_th;
-        const bool gb = xtra && s_q[b + 32] >= P.q_th;
-        float4 na, nb;
-        if (ga || gb) {
-          const long long row = s_row[r];
-          if (ga) na = __ldg(nrm + row + xl);
-          if (gb) nb = __ldg(nrm + row + xr);
-        }
-        if (ga) {
-          s_n[b] = na.x; s_n[G::NB + b] = na.y; s_n[2 * G::NB + b] = na.z;
-          lo0 = fminf(lo0, na.x); lo1 = fminf(lo1, na.y); lo2 = fminf(lo2, na.z);
-          hi0 = fmaxf(hi0, na.x); hi1 = fmaxf(hi1, na.y); hi2 = fmaxf(hi2, na.z);
-        } else {
-          s_n[b] = s_n[G::NB + b] = s_n[2 * G::NB + b] = qnan;
-        }
-        if (xtra) {
-          if (gb) {
-            s_n[b + 32] = nb.x; s_n[G::NB + b + 32] = nb.y; s_n[2 * G::NB + b + 32] = nb.z;
-            lo0 = fminf(lo0, nb.x); lo1 = fminf(lo1, nb.y); lo2 = fminf(lo2, nb.z);
-            hi0 = fmaxf(hi0, nb.x); hi1 = fmaxf(hi1, nb.y); hi2 = fmaxf(hi2, nb.z);
-          } else {
-            s_n[b + 32] = s_n[G::NB + b + 32] = s_n[2 * G::NB + b + 32] = qnan;
-          }
-        }
-      }
-    }
-#pragma unroll
-    for (int sh = 16; sh > 0; sh >>= 1) {
-      lo0 = fminf(lo0, __shfl_xor_sync(0xffffffffu, lo0, sh));
-      lo1 = fminf(lo1, __shfl_xor_sync(0xffffffffu, lo1, sh));
-      lo2 = fminf(lo2, __shfl_xor_sync(0xffffffffu, lo2, sh));
-      hi0 = fmaxf(hi0, __shfl_xor_sync(0xffffffffu, hi0, sh));
-      hi1 = fmaxf(hi1, __shfl_xor_sync(0xffffffffu, hi1, sh));
-      hi2 = fmaxf(hi2, __shfl_xor_sync(0xffffffffu, hi2, sh));
-    }
-    if (lane == 0) {
-      float *rw = s_rng + 6 * warp;
-      rw[0] = lo0; rw[1] = lo1; rw[2] = lo2; rw[3] = hi0; rw[4] = hi1; rw[5] = hi2;
-    }
-    if (tid == 0) *s_count = 0;
+    const int32_t v = phi[idx];
+    const float4 nv = __ldg(nrm + idx);  // used where gated
+    for (int i = tid; i < kClasses<DIM> * M::ROWS; i += G::NT) (&s_box.m[0][0])[i] = make_uint2(0u, 0u);
+    if (tid == 0) s_count = 0;
     __syncthreads();
-    if (tid < 6) {
-      float a = s_rng[tid];
-      for (int w = 1; w < G::NW; w++) a = tid < 3 ? fminf(a, s_rng[6 * w + tid]) : fmaxf(a, s_rng[6 * w + tid]);
-      s_rng[6 * G::NW + tid] = a;
-    }
-    __syncthreads();
-    const float rlo0 = s_rng[6 * G::NW], rlo1 = s_rng[6 * G::NW + 1], rlo2 = s_rng[6 * G::NW + 2];
-    const float rhi0 = s_rng[6 * G::NW + 3], rhi1 = s_rng[6 * G::NW + 4], rhi2 = s_rng[6 * G::NW + 5];
-    const float thr = P.cos_opp + 1e-5f;
-    const int ob0 = (DIM == 3 ? (tz + G::H) * G::HX * G::HY : 0) + (ty + G::H) * G::HX + tx + G::H;
-    if (tiles) gated = inb && s_q[ob0] >= P.q_th;
-    bool scan = false;
-    if (gated) {
-      const float n0 = s_n[ob0], n1 = s_n[G::NB + ob0], n2 = s_n[2 * G::NB + ob0];
-      scan = fminf(n0 * rlo0, n0 * rhi0) + fminf(n1 * rlo1, n1 * rhi1) + fminf(n2 * rlo2, n2 * rhi2) <= thr;
-    }
-    if (__syncthreads_or(scan)) {
-      // window ranges: z pass (3D) over the box columns, y pass, then x per cell
-      if constexpr (DIM == 3) {
-        for (int col = tid; col < G::HX * G::HY; col += G::NT) {
-#pragma unroll
-          for (int a = 0; a < 3; a++) {
-            float v[G::HZ];
-#pragma unroll
-            for (int k = 0; k < G::HZ; k++) v[k] = s_n[a * G::NB + k * G::HX * G::HY + col];
-            static_assert(G::HZ == 10 && G::TZ == 4, "window filter of four outputs over ten planes");
-            float lo[4], hi[4];
-            win7x4<false>(v, lo);
-            win7x4<true>(v, hi);
-#pragma unroll
-            for (int o = 0; o < G::TZ; o++) {
-              s_zr[(2 * a) * G::NZR + o * G::HX * G::HY + col] = __float2half_rd(lo[o]);
-              s_zr[(2 * a + 1) * G::NZR + o * G::HX * G::HY + col] = __float2half_ru(hi[o]);
-            }
-          }
-        }
-        __syncthreads();
-      }
-      for (int col = tid; col < G::HX * G::TZ; col += G::NT) {
-        const int cx = col % G::HX, cz = col / G::HX;
-#pragma unroll
-        for (int c = 0; c < 6; c++) {
-          float v[G::HY];
-#pragma unroll
-          for (int k = 0; k < G::HY; k++) {
-            if constexpr (DIM == 3) {
-              v[k] = __half2float(s_zr[c * G::NZR + (cz * G::HY + k) * G::HX + cx]);
-            } else {
-              v[k] = s_n[(c >> 1) * G::NB + k * G::HX + cx];
-            }
-          }
-          if constexpr (G::HY == 10 && G::TY == 4) {
-            float r[4];
-            if (c & 1) win7x4<true>(v, r); else win7x4<false>(v, r);
-#pragma unroll
-            for (int o = 0; o < G::TY; o++)
-              s_yr[c * G::NYR + (cz * G::TY + o) * G::HX + cx] = (c & 1) ? __float2half_ru(r[o]) : __float2half_rd(r[o]);
-          } else if constexpr (G::HY == 14 && G::TY == 8) {
-            float r[8];
-            if (c & 1) win7x8<true>(v, r); else win7x8<false>(v, r);
-#pragma unroll
-            for (int o = 0; o < G::TY; o++)
-              s_yr[c * G::NYR + (cz * G::TY + o) * G::HX + cx] = (c & 1) ? __float2half_ru(r[o]) : __float2half_rd(r[o]);
-          } else {
-#pragma unroll
-            for (int o = 0; o < G::TY; o++) {
-              float r = v[o];
-#pragma unroll
-              for (int k = 1; k <= 2 * G::H; k++) r = (c & 1) ? fmaxf(r, v[o + k]) : fminf(r, v[o + k]);
-              s_yr[c * G::NYR + (cz * G::TY + o) * G::HX + cx] = (c & 1) ? __float2half_ru(r) : __float2half_rd(r);
-            }
-          }
-        }
-      }
-      __syncthreads();
-      if (scan) {
-        const __half *row = s_yr + (tz * G::TY + ty) * G::HX + tx;
-        float b = 0.0f;
-#pragma unroll
-        for (int a = 0; a < 3; a++) {
-          float lo = __half2float(row[(2 * a) * G::NYR]), hi = __half2float(row[(2 * a + 1) * G::NYR]);
-#pragma unroll
-          for (int k = 1; k <= 2 * G::H; k++) {
-            lo = fminf(lo, __half2float(row[(2 * a) * G::NYR + k]));
-            hi = fmaxf(hi, __half2float(row[(2 * a + 1) * G::NYR + k]));
-          }
-          const float na = s_n[a * G::NB + ob0];
-          b += fminf(na * lo, na * hi);
-        }
-        scan = b <= thr;
-      }
-    }
-    if (gated && !scan) {  // no candidate can face this cell: no force
+    stage_masks<DIM>(P, s_box, masks, mark, gtx, gty, x0, y0, z0, tid, G::NT);
+    const bool gated = inb && q_gate_value(v) >= P.q_th;
+    if (!list && inb && ((tx + ty + tz) & (parts - 1)) == part) {
       frep[idx] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (partner) partner[3 * idx] = partner[3 * idx + 1] = partner[3 * idx + 2] = INT32_MIN;
     }
-    {  // compact the cells to scan
+    __syncthreads();
+    {  // list the cells with a possible partner
+      const bool scan = gated && ((tx + ty + tz) & (parts - 1)) == part && may_face<DIM, W>(s_box, nv, tx, ty, tz);
       const unsigned m = __ballot_sync(0xffffffffu, scan);
       int base = 0;
-      if (lane == 0 && m) base = atomicAdd(s_count, __popc(m));
+      if (lane == 0 && m) base = atomicAdd(&s_count, __popc(m));
       base = __shfl_sync(0xffffffffu, base, 0);
-      if (scan) s_list[base + __popc(m & ((1u << lane) - 1u))] = tid;
-    }
-    if (debug && inb && !gated) {
-      frep[idx] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (partner) partner[3 * idx] = partner[3 * idx + 1] = partner[3 * idx + 2] = INT32_MIN;
+      if (scan) {
+        const int k = base + __popc(m & ((1u << lane) - 1u));
+        s_list[k] = tid;
+        s_n[k] = nv;
+        s_v[k] = v;
+      }
     }
     __syncthreads();
-
-    // one warp per gated cell; candidate criteria Eqs. 59, 61, 62; the winner is the nearest
-    // accepted candidate, then the largest facing score, then the first in table order (the
-    // packed key orders exactly that way)
-    const int ncell = *s_count;
+    const int ncell = s_count;
     for (int k = warp; k < ncell; k += G::NW) {
       const int c = s_list[k];
       const int cx = c % G::TX, cy = (c / G::TX) % G::TY, cz = c / (G::TX * G::TY);
-      const int ob = (DIM == 3 ? (cz + G::H) * G::HX * G::HY : 0) + (cy + G::H) * G::HX + cx + G::H;
-      const int32_t vx = s_phi[ob];
-      const float qxc = s_q[ob];
-      const float n0 = s_n[ob], n1 = s_n[G::NB + ob], n2 = s_n[2 * G::NB + ob];
-      unsigned long long best = ~0ull;
-      {
-        const float sim = __fmul_rn(P.eta, fmaxf(qxc, P.eps_q));
-        for (int j0 = 0; j0 < T.count; j0 += 32) {
-          // stop once a candidate is held and this chunk starts beyond its shell
-          if (best != ~0ull && (int)T.o[j0].d2 > (int)(best >> 40)) break;
-          const int j = j0 + lane;
-          unsigned long long key = ~0ull;
-          if (j < T.count) {
-            const NciOffset o = T.o[j];
-            const int yb = ob + o.dx + G::HX * (o.dy + G::HY * o.dz);
-            const float qy = s_q[yb];
-            if (qy >= P.q_th && fabsf(__fsub_rn(qy, qxc)) <= sim) {
-              const float dot = __fadd_rn(__fadd_rn(__fmul_rn(n0, s_n[yb]), __fmul_rn(n1, s_n[G::NB + yb])),
-                                          __fmul_rn(n2, s_n[2 * G::NB + yb]));
-              if (dot <= P.cos_opp) {
-                const float ff = fmaxf(-dot, 0.0f);
-                key = ((unsigned long long)o.d2 << 40) |
-                      ((unsigned long long)(0x7fffffffu - __float_as_uint(ff)) << 9) | (unsigned long long)j;
-              }
-            }
-          }
-          if (__any_sync(0xffffffffu, key != ~0ull)) {
-#pragma unroll
-            for (int sh = 16; sh > 0; sh >>= 1) {
-              const unsigned long long other = __shfl_xor_sync(0xffffffffu, key, sh);
-              key = other < key ? other : key;
-            }
-            best = key < best ? key : best;
-          }
-        }
-      }
-      if (lane != 0) continue;
-      const long long gidx = (long long)(x0 + cx) + (long long)nx * ((y0 + cy) + (long long)ny * (z0 + cz));
-      float4 out = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (best != ~0ull) {
-        const int bj = (int)(best & 511ull);
-        const NciOffset o = T.o[bj];
-        const float ff = __uint_as_float(0x7fffffffu - (unsigned)((best >> 9) & 0x7fffffffull));
-        const int yb = ob + o.dx + G::HX * (o.dy + G::HY * o.dz);
-        const int32_t vy = s_phi[yb];
-        const float m0 = s_n[yb], m1 = s_n[G::NB + yb], m2 = s_n[2 * G::NB + yb];
-        const float qy = s_q[yb];
-        // paired indicator and clamp, Eqs. 66-67
-        const float qpair = 0.5f * (qxc + qy);
-        const float qcl = fminf(fmaxf(qpair, P.eps_q), 0.25f - P.eps_q);
-        // proximity indicator, Eq. 70, as eps * artanh(sqrt(1 - 4 q)): the same value, and
-        // 1 - 4 q_pair = ((1 - 2 phi_x)^2 + (1 - 2 phi_y)^2) / 2 has no cancellation
-        float mm;
-        if (qcl == qpair) {
-          const float ax = 1.0f - 2.0f * fminf(fmaxf(phi_of(vx), 0.f), 1.f);
-          const float ay = 1.0f - 2.0f * fminf(fmaxf(phi_of(vy), 0.f), 1.f);
-          mm = 0.5f * (ax * ax + ay * ay);
-        } else {
-          mm = 1.0f - 4.0f * qcl;
-        }
-        const float h = P.eps * atanhf(sqrtf(mm));
-        const float tt = h / P.h0;
-        const float tp = (P.p == 4.0f) ? (tt * tt) * (tt * tt) : powf(tt, P.p);
-        const float wh = 1.0f / (1.0f + tp);  // Eq. 71
-        // symmetric normal, Eq. 69, line-of-centres fallback, oriented toward the partner
-        const float rn = sqrtf((float)o.d2);
-        const float r0 = o.dx / rn, r1 = o.dy / rn, r2 = o.dz / rn;
-        float s0 = n0 - m0, s1 = n1 - m1, s2 = n2 - m2;
-        const float sn = sqrtf(s0 * s0 + s1 * s1 + s2 * s2);
-        if (sn < 1e-8f) {
-          s0 = r0; s1 = r1; s2 = r2;
-        } else {
-          const float is = 1.0f / (sn + P.eps_n);
-          s0 *= is; s1 *= is; s2 *= is;
-        }
-        if (r0 * s0 + r1 * s1 + r2 * s2 < 0.0f) {
-          s0 = -s0; s1 = -s1; s2 = -s2;
-        }
-        // flux and force density with the facing factor of Eq. 68, Eqs. 72-73
-        const float rho = P.rho_g + P.drho * phi_of(vx);
-        const float amp = rho * P.A_rep * qcl * wh * ff;
-        out = make_float4(amp * s0, amp * s1, DIM == 3 ? amp * s2 : 0.0f, 1.0f);
-        if (partner) {
-          partner[3 * gidx] = o.dx;
-          partner[3 * gidx + 1] = o.dy;
-          partner[3 * gidx + 2] = o.dz;
-        }
-      } else if (partner) {
-        partner[3 * gidx] = partner[3 * gidx + 1] = partner[3 * gidx + 2] = INT32_MIN;
-      }
-      frep[gidx] = out;
+      const float4 me = s_n[k];
+      const unsigned long long best =
+          pair_of<DIM, W>(P, phi, nrm, x0 + cx, y0 + cy, z0 + cz, me, s_v[k], lane,
+                          s_box.m[facing_class<DIM>(me)] + (DIM == 3 ? (cz + kWin) * M::HY : 0) + cy + kWin, cx, s_cand[warp]);
+      if (lane == 0) s_best[k] = best;
     }
-    __syncthreads();  // the next tile reuses the shared buffers
+    __syncthreads();
+    if (tid < ncell && s_best[tid] != ~0ull) {  // a thread per cell; without a partner the force stays zero
+      const int c = s_list[tid];
+      pair_force<DIM, W>(P, phi, nrm, frep, partner, x0 + c % G::TX, y0 + (c / G::TX) % G::TY, z0 + c / (G::TX * G::TY),
+                         s_n[tid], s_v[tid], s_best[tid]);
+    }
+    __syncthreads();  // the next unit reuses the shared buffers
   }
 }
 
 template <int DIM>
-static cudaError_t nci_attr() {
+static cudaError_t launch_nci_dim(const KParams &P, const int32_t *phi, float4 *nrm, float4 *frep, int32_t *partner,
+                                  const TileList &list, int list_blocks, cudaStream_t s, const NciAux &aux,
+                                  int *reset_other, int max_parts) {
   using G = NciGeom<DIM>;
-  static bool done = false;
-  if (done) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(k_nci_scan<DIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::smem);
-  if (e == cudaSuccess) done = true;
-  return e;
-}
-
-template <int DIM>
-static cudaError_t launch_nci_dim(const KParams &P, const NciTable &T, const int32_t *phi, float4 *nrm, float4 *frep,
-                                  int32_t *partner, int debug, const int *tiles, const int *ntiles, int list_blocks,
-                                  cudaStream_t s, const NciAux *aux, int *reset_other) {
-  using G = NciGeom<DIM>;
-  cudaError_t e = nci_attr<DIM>();
-  if (e != cudaSuccess) return e;
-  const int gtx = (P.nx + G::TX - 1) / G::TX, gty = (P.ny + G::TY - 1) / G::TY, gtz = (P.nz + G::TZ - 1) / G::TZ;
-  const int total = gtx * gty * gtz;
-  // resident blocks walk the list; a small grid has fewer tiles than that
-  const int blocks = tiles ? (total < list_blocks ? total : list_blocks) : (total < list_blocks * 4 ? total : list_blocks * 4);
-  dim3 block(G::TX, G::TY, G::TZ);
-  const bool pre = DIM == 3 && aux && tiles && aux->bricks && nci_aux_applies(DIM, P);
-  const NciAux none{};
+  const int *tiles = list.tiles, *ntiles = list.count;
+  const int gtx = (P.nx + NciTile<DIM>::X - 1) / NciTile<DIM>::X, gty = (P.ny + NciTile<DIM>::Y - 1) / NciTile<DIM>::Y,
+            gtz = (P.nz + NciTile<DIM>::Z - 1) / NciTile<DIM>::Z;
+  const int total = gtx * gty * gtz, units = G::UNITS * total;
+  // grid-stride blocks walk the lists, at most 16 (normals, prefilter) or 2 (scan) per list block; a small
+  // grid has fewer items than that
+  const int most = 16 * list_blocks, scan_blocks = units < 2 * list_blocks ? units : 2 * list_blocks;
+  const dim3 block(G::TX, G::TY, G::TZ);
+  int *reset = tiles ? reset_other : nullptr;
+  cudaError_t e;
   if constexpr (DIM == 2) {
-    cudaError_t e2 = launch_pdl(k_nci_normals2, dim3(blocks), block, 0, s, P, phi, nrm, tiles, ntiles, total, gtx, gty,
-                                tiles ? reset_other : nullptr);
-    if (e2 != cudaSuccess) return e2;
+    e = launch_pdl(k_nci_normals2, dim3(total < most ? total : most), block, 0, s, P, phi, nrm, frep, tiles, ntiles, total,
+                   gtx, gty, aux.masks, reset);
   } else {
-    // one block per half tile, at most 16 blocks per resident scan block (grid-stride beyond)
-    const int nb = 2 * total < 16 * list_blocks ? 2 * total : 16 * list_blocks;
-    cudaError_t e3 = launch_pdl(k_nci_normals3, dim3(nb), dim3(kNrmThreads), 0, s, P, phi, nrm, frep, tiles, ntiles, total,
-                                gtx, gty, pre ? *aux : none, tiles ? reset_other : nullptr);
-    if (e3 != cudaSuccess) return e3;
+    NciAux a = aux;
+    if (!tiles) a.bricks = nullptr;
+    e = launch_pdl(k_nci_normals3, dim3(2 * total < most ? 2 * total : most), dim3(kNrmThreads), 0, s, P, phi, nrm, frep,
+                   tiles, ntiles, total, gtx, gty, a, reset);
   }
-  if (!pre) {
-    return launch_pdl(k_nci_scan<DIM>, dim3(blocks), block, G::smem, s, P, T, phi, nrm, frep, partner, debug, tiles,
-                      ntiles, total, gtx, gty, nullptr, nullptr, nullptr);
-  }
-  e = launch_pdl(k_nci_prefilter, dim3(total < 16 * list_blocks ? total : 16 * list_blocks), dim3(128), 0, s, P,
-                 (const uint4 *)aux->bricks,
-                 (const unsigned char *)aux->flags, tiles, ntiles, aux->scan_tiles, aux->nscan, gtx, gty);
   if (e != cudaSuccess) return e;
-  return launch_pdl(k_nci_scan<DIM>, dim3(blocks), block, G::smem, s, P, T, phi, nrm, frep, partner, debug,
-                    (const int *)aux->scan_tiles, (const int *)aux->nscan, total, gtx, gty, aux->flags, tiles, ntiles);
+  const unsigned *masks = aux.masks;
+  const float4 *normals = nrm;
+  const uint4 *bricks = nullptr;
+  const int *mark = tiles ? list.mark : nullptr, *items = tiles, *count = ntiles;
+  bool per_tile = tiles != nullptr;
+  if (tiles && nci_prefilter_applies(DIM, P)) {
+    e = launch_pdl(k_nci_prefilter, dim3(total < most ? total : most), dim3(128), 0, s, P, aux, mark, tiles, ntiles, gtx,
+                   gty);
+    if (e != cudaSuccess) return e;
+    items = aux.scan_units;
+    count = aux.nscan;
+    per_tile = false;
+  } else if (tiles) {
+    // Where a side is not a multiple of 4 an entry of the brick test reads several bricks, and the test is
+    // made by the scan's own blocks: the pass has no prefilter kernel.
+    bricks = aux.bricks;
+  }
+  const auto scan = P.w == 3 ? k_nci_scan<DIM, 3> : (P.w == 2 ? k_nci_scan<DIM, 2> : k_nci_scan<DIM, 1>);
+  return launch_pdl(scan, dim3(scan_blocks), block, 0, s, P, phi, normals, frep, partner, items, count, per_tile, units,
+                    gtx, gty, masks, bricks, mark, max_parts);
 }
 
-cudaError_t launch_nci(int dim, const KParams &P, const NciTable &T, const int32_t *phi, float4 *nrm, float4 *frep,
-                       int32_t *partner, int debug, const int *tiles, const int *ntiles, int list_blocks,
-                       cudaStream_t s, const NciAux *aux, int *reset_other) {
-  return dim == 2 ? launch_nci_dim<2>(P, T, phi, nrm, frep, partner, debug, tiles, ntiles, list_blocks, s, aux,
-                                      reset_other)
-                  : launch_nci_dim<3>(P, T, phi, nrm, frep, partner, debug, tiles, ntiles, list_blocks, s, aux,
-                                      reset_other);
+cudaError_t launch_nci(int dim, const KParams &P, const int32_t *phi, float4 *nrm, float4 *frep, int32_t *partner,
+                       const TileList &list, int list_blocks, cudaStream_t s, const NciAux &aux, int *reset_other,
+                       int max_parts) {
+  return dim == 2 ? launch_nci_dim<2>(P, phi, nrm, frep, partner, list, list_blocks, s, aux, reset_other, max_parts)
+                  : launch_nci_dim<3>(P, phi, nrm, frep, partner, list, list_blocks, s, aux, reset_other, max_parts);
 }
 
-bool nci_aux_applies(int dim, const KParams &P) {
+bool nci_prefilter_applies(int dim, const KParams &P) {
   return dim == 3 && P.nx % 4 == 0 && P.ny % 4 == 0 && P.nz % 4 == 0;
 }
 
-size_t nci_brick_count(const KParams &P) { return (size_t)(P.nx / 4) * (size_t)(P.ny / 4) * (size_t)(P.nz / 4); }
+size_t nci_brick_count(const KParams &P) {
+  return (size_t)((P.nx + 3) / 4) * (size_t)((P.ny + 3) / 4) * (size_t)((P.nz + 3) / 4);
+}
 
-int nci_list_blocks(int dim) {
-  int dev = 0, sms = 0, per = 0;
+size_t nci_mask_bytes(const KParams &P) {
+  return sizeof(unsigned) * kMaskWords * (size_t)((P.nx + 31) / 32) * (size_t)P.ny * (size_t)P.nz;
+}
+
+// SMs of the device: the near-contact kernels are launched with a number of blocks per SM.
+int nci_list_blocks() {
+  int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-  if (dim == 2) {
-    if (nci_attr<2>() != cudaSuccess) return 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_nci_scan<2>, NciGeom<2>::NT, NciGeom<2>::smem);
-  } else {
-    if (nci_attr<3>() != cudaSuccess) return 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_nci_scan<3>, NciGeom<3>::NT, NciGeom<3>::smem);
-  }
-  return sms * (per > 0 ? per : 1);
+  return sms;
 }
 
 }  // namespace lbm

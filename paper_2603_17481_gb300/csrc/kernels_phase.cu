@@ -132,7 +132,7 @@ __device__ __forceinline__ int32_t face_transfer(const KParams &P, const int32_t
 template <int DIM>
 __global__ void __launch_bounds__(PhaseGeom<DIM>::NT)
 k_phase(const KParams P, const int32_t *__restrict__ phi, const float *__restrict__ u,
-        int32_t *__restrict__ phi_out, int *__restrict__ tiles, int *__restrict__ ntiles) {
+        int32_t *__restrict__ phi_out, const TileList next) {
   pdl_enter();
   using G = PhaseGeom<DIM>;
   using SL = typename StencilOf<DIM>::type;
@@ -219,22 +219,23 @@ k_phase(const KParams P, const int32_t *__restrict__ phi, const float *__restric
     phi_out[(long long)x + (long long)nx * (y + (long long)ny * z)] = vn;
     gated = q_gate_value(vn) >= P.q_th;
   }
-  if (tiles) {
+  if (next.tiles) {  // one block per tile: it sets the tile's mark either way
     const int any = __syncthreads_or(gated);
-    if (any && tid == 0) {
+    if (tid == 0) {
       const int tile = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-      tiles[atomicAdd(ntiles, 1)] = tile;
+      next.mark[tile] = any != 0;
+      if (any) next.tiles[atomicAdd(next.count, 1)] = tile;
     }
   }
 }
 
 template <int DIM>
 static cudaError_t launch_phase_dim(const KParams &P, const int32_t *phi, const float *u, int32_t *phi_out,
-                                    int *tiles, int *ntiles, cudaStream_t s) {
+                                    const TileList &next, cudaStream_t s) {
   using G = PhaseGeom<DIM>;
   dim3 block(G::TX, G::TY, G::TZ);
   dim3 grid((P.nx + G::TX - 1) / G::TX, (P.ny + G::TY - 1) / G::TY, (P.nz + G::TZ - 1) / G::TZ);
-  return launch_pdl(k_phase<DIM>, grid, block, 0, s, P, phi, u, phi_out, tiles, ntiles);
+  return launch_pdl(k_phase<DIM>, grid, block, 0, s, P, phi, u, phi_out, next);
 }
 
 // Records once, at context creation, how many k_phase3m blocks the device holds at once (SMs x
@@ -279,7 +280,7 @@ static cudaError_t launch_phase3(const KParams &P, const int32_t *phi, const flo
 
 cudaError_t launch_phase(int dim, const KParams &P, const int32_t *phi, const float *u, int32_t *phi_out,
                          const TileList &next, const TileList &prev, cudaStream_t s) {
-  return dim == 2 ? launch_phase_dim<2>(P, phi, u, phi_out, next.tiles, next.count, s)
+  return dim == 2 ? launch_phase_dim<2>(P, phi, u, phi_out, next, s)
                   : launch_phase3(P, phi, u, phi_out, next, prev, s);
 }
 
@@ -298,7 +299,7 @@ k_gate_tiles(const KParams P, const int32_t *__restrict__ phi, int *__restrict__
   if (any && threadIdx.x == 0 && threadIdx.y == 0 && threadIdx.z == 0) {
     const int tile = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
     tiles[atomicAdd(ntiles, 1)] = tile;
-    if (mark) mark[tile] = 1;
+    mark[tile] = 1;
   }
 }
 
@@ -306,7 +307,7 @@ cudaError_t launch_gate_tiles(int dim, const KParams &P, const int32_t *phi, con
   if (dim == 2) {
     using G = PhaseGeom<2>;
     dim3 grid((P.nx + G::TX - 1) / G::TX, (P.ny + G::TY - 1) / G::TY, 1);
-    k_gate_tiles<2><<<grid, dim3(G::TX, G::TY, G::TZ), 0, s>>>(P, phi, list.tiles, list.count, nullptr);
+    k_gate_tiles<2><<<grid, dim3(G::TX, G::TY, G::TZ), 0, s>>>(P, phi, list.tiles, list.count, list.mark);
   } else {
     using G = PhaseGeom<3>;
     dim3 grid((P.nx + G::TX - 1) / G::TX, (P.ny + G::TY - 1) / G::TY, (P.nz + G::TZ - 1) / G::TZ);

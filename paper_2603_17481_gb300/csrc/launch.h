@@ -23,40 +23,46 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
-// Window offsets of the near-contact search, sorted by (|r|^2, canonical index), passed by value.
-struct NciTable {
-  NciOffset o[kMaxOffsets];
-  int count;
-};
-
 // Kernel modes of the hydrodynamic kernel.
 enum HydroMode { kStep = 0, kMoments = 1 };
 
-// Buffers of the near-contact prefilter (3D grids whose sides are multiples of 4): the component
-// ranges of the gated normals of every 4x4x4 brick, as halves lo0 lo1 lo2 - hi0 hi1 hi2 - (lo
-// rounded down, hi up); a flag per tile, set while the tile is listed for the current phi (zero
-// between steps); the listed tiles that may hold a facing pair, and their count.
+// The near-contact list of one phi buffer: the 32 x 8 x 4 tiles (3D; 32 x 16 in 2D) holding a
+// gated cell, their count, and one mark per tile of the grid, set while the tile is listed.
+struct TileList {
+  int *tiles = nullptr;
+  int *count = nullptr;
+  int *mark = nullptr;
+};
+
+// Buffers of the near-contact pass besides the normals and forces: for every row of 32 cells of a
+// listed tile the masks of its gated cells by the direction of their normals (8 words, 6 or 4 used);
+// in 3D the component ranges of the gated normals of every 4x4x4 brick, as halves lo0 lo1 lo2 - hi0
+// hi1 hi2 - (lo rounded down, hi up); the half tiles that may hold a facing pair (2 * tile + half),
+// and their count.
 struct NciAux {
+  unsigned *masks = nullptr;
   uint4 *bricks = nullptr;
-  unsigned char *flags = nullptr;
-  int *scan_tiles = nullptr;
+  int *scan_units = nullptr;
   int *nscan = nullptr;
 };
-bool nci_aux_applies(int dim, const KParams &P);
+bool nci_prefilter_applies(int dim, const KParams &P);
 size_t nci_brick_count(const KParams &P);
+size_t nci_mask_bytes(const KParams &P);
 
-// Normals of the gated cells into nrm, then the window scan writing frep at gated cells.
-// tiles == nullptr: every tile (debug = 1 also writes zero force / no partner at every cell);
-// otherwise only the ntiles listed tiles, walked by list_blocks resident blocks. With aux (listed
-// tiles only), the normals pass also writes zero force at every gated cell and the brick ranges,
-// a prefilter keeps the tiles whose bricks may face another interface, and only those are scanned.
+// Most blocks that share one scanned unit (1 where several cases share the device).
+constexpr int kNciParts = 8;
+
+// The near-contact pass over the listed tiles on phi: normals of the gated cells into nrm, zero force
+// at them, then the force at the cells that have a partner. list.tiles == nullptr: over every tile, with
+// zero force (and no partner, where partner is given) at every other cell too.
+// list_blocks: blocks per kernel are at most a few times this (the device's SMs, or fewer).
 // reset_other (listed tiles, may be null): the count of the other phi buffer's list, whose tiles
 // were consumed by the previous step; the normals pass sets it to zero, so that the phase pass of
 // this step starts that buffer's list empty.
-cudaError_t launch_nci(int dim, const KParams &P, const NciTable &T, const int32_t *phi, float4 *nrm, float4 *frep,
-                       int32_t *partner, int debug, const int *tiles, const int *ntiles, int list_blocks,
-                       cudaStream_t s, const NciAux *aux = nullptr, int *reset_other = nullptr);
-int nci_list_blocks(int dim);
+cudaError_t launch_nci(int dim, const KParams &P, const int32_t *phi, float4 *nrm, float4 *frep, int32_t *partner,
+                       const TileList &list, int list_blocks, cudaStream_t s, const NciAux &aux,
+                       int *reset_other = nullptr, int max_parts = kNciParts);
+int nci_list_blocks();
 cudaError_t phase_prepare(int dim);
 
 // src/dst are population buffers of the store type; MODE kStep writes dst and u, kMoments writes
@@ -68,14 +74,6 @@ cudaError_t launch_hydro(int Q, int store, int mode, const KParams &P, const voi
 #ifndef LBM_HYDRO2_MINB
 #define LBM_HYDRO2_MINB 3
 #endif
-
-// The near-contact list of one phi buffer: the 32 x 8 x 4 tiles (3D; 32 x 8 in 2D) holding a
-// gated cell, their count, and one mark per tile of the grid (3D), set while the tile is listed.
-struct TileList {
-  int *tiles = nullptr;
-  int *count = nullptr;
-  int *mark = nullptr;
-};
 
 // The hydrodynamic step split in two launches around the near-contact pass (3D, nx even,
 // Q N <= 2^32: the paired kernel). part 0 updates every 64 x 2 x 2 tile half whose near-contact

@@ -100,32 +100,21 @@ void derive_kparams(const lbm_params &p, KParams &K) {
   K.rho_bar = (float)p.rho_l;
   for (int a = 0; a < 3; a++) K.g[a] = (float)p.g[a];
   K.nci_on = p.nci_on;
-  K.w = p.w;
+  K.w = p.nci_on ? p.w : 1;
   K.A_rep = (float)p.A_rep; K.h0 = (float)p.h0; K.p = (float)p.p; K.q_th = (float)p.q_th;
   K.eta = (float)p.eta; K.cos_opp = (float)p.cos_opp; K.eps_q = (float)p.eps_q; K.eps_n = (float)p.eps_n;
   K.eps = (float)p.eps;
   K.Dlap = (float)(p.D * 6.0);
   K.kc = (float)(3.0 * 4.0 * p.D / p.eps);
+  // The largest m_a of a normal m (|m| <= 1) with n.m <= cos_opp < 0, for any n (|n| <= 1) whose largest
+  // component is n_a > 0: n.m >= n_a m_a - |n_t| sqrt(1 - m_a^2) with n_a >= |n| / sqrt(3), which is at most
+  // cos_opp only if m_a <= sin(psi), -cos(psi + asin(1 / sqrt(3))) = cos_opp (or m_a <= 0 where psi < 0). The
+  // margin covers the rounding of the normals, their lengths and their product. With cos_opp >= 0 a
+  // short normal may be paired with any other.
+  const double psi = std::acos(std::min(1.0, std::max(-1.0, -p.cos_opp))) - std::asin(1.0 / std::sqrt(3.0));
+  K.face_t = p.cos_opp < 0.0 ? (float)(std::sin(std::max(0.0, psi)) + 2e-3) : 2.0f;
   K.rho_g64 = p.rho_g;
   K.drho64 = p.rho_l - p.rho_g;
-}
-
-// Window offsets of Eq. 60 sorted by |r|^2, then by the canonical index
-// ((rz + w)(2w + 1) + (ry + w))(2w + 1) + (rx + w).
-void build_table(int dim, int w, NciTable &T) {
-  struct E { int d2, k, dx, dy, dz; };
-  std::vector<E> v;
-  const int W = 2 * w + 1, zr = dim == 3 ? w : 0;
-  for (int rz = -zr; rz <= zr; rz++)
-    for (int ry = -w; ry <= w; ry++)
-      for (int rx = -w; rx <= w; rx++) {
-        if (!rx && !ry && !rz) continue;
-        v.push_back({rx * rx + ry * ry + rz * rz, ((rz + zr) * W + (ry + w)) * W + (rx + w), rx, ry, rz});
-      }
-  std::sort(v.begin(), v.end(), [](const E &a, const E &b) { return a.d2 != b.d2 ? a.d2 < b.d2 : a.k < b.k; });
-  T.count = (int)v.size();
-  for (int i = 0; i < T.count; i++)
-    T.o[i] = NciOffset{(int8_t)v[i].dx, (int8_t)v[i].dy, (int8_t)v[i].dz, (int8_t)v[i].d2};
 }
 
 // bytes of one population buffer
@@ -246,8 +235,8 @@ int run_moments(lbm_ctx *c) {
   const int d = c->P.dim;
   if (c->P.nci_on) {
     rc = from_cuda(timed(c, LBM_K_NCI, [&] {
-      return launch_nci(d, c->K, c->T, c->phi[c->pcur], c->nrm, c->frep, nullptr, 0, c->tiles[c->pcur],
-                        c->ntiles + c->pcur, c->nci_blocks, c->stream, nci_aux(c), c->ntiles + (c->pcur ^ 1));
+      return launch_nci(d, c->K, c->phi[c->pcur], c->nrm, c->frep, nullptr, tile_list(c, c->pcur),
+                        c->nci_blocks, c->stream, c->aux, c->ntiles + (c->pcur ^ 1));
     }, nci_list_kernels(c)));
     if (rc) return rc;
   }
@@ -265,7 +254,7 @@ int run_moments(lbm_ctx *c) {
 // phase-field pass. With lists, the phase-field pass lists the tiles of phi^{n+1} and clears the
 // marks of phi^n's list; without, the lists are left as they are (a dry step writes only the
 // next-step buffers and per-step scratch). Makes no non-stream CUDA call (it may be captured).
-int enqueue_step(lbm_ctx *c, int cur, int pcur, bool lists, cudaStream_t st) {
+int enqueue_step(lbm_ctx *c, int cur, int pcur, bool lists, cudaStream_t st, int nci_parts) {
   const int d = c->P.dim, nxt = cur ^ 1, pn = pcur ^ 1;
   const bool nci = c->P.nci_on != 0;
   int rc;
@@ -277,8 +266,8 @@ int enqueue_step(lbm_ctx *c, int cur, int pcur, bool lists, cudaStream_t st) {
     if (!rc) rc = from_cuda(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
     if (rc) return rc;
     rc = from_cuda(timed_on(c, c->side, LBM_K_NCI, [&] {
-      return launch_nci(d, c->K, c->T, c->phi[pcur], c->nrm, c->frep, nullptr, 0, c->tiles[pcur], c->ntiles + pcur,
-                        c->overlap_blocks, c->side, nci_aux(c), c->ntiles + pn);
+      return launch_nci(d, c->K, c->phi[pcur], c->nrm, c->frep, nullptr, listed, c->overlap_blocks, c->side,
+                        c->aux, c->ntiles + pn, nci_parts);
     }, nci_list_kernels(c)));
     if (rc) return rc;
     rc = from_cuda(launch_hydro_split(1, c->P.Q, c->P.store, c->K, c->pop[cur], c->pop[nxt], c->phi[pcur], c->frep,
@@ -296,8 +285,8 @@ int enqueue_step(lbm_ctx *c, int cur, int pcur, bool lists, cudaStream_t st) {
   } else {
     if (nci) {
       rc = from_cuda(timed_on(c, st, LBM_K_NCI, [&] {
-        return launch_nci(d, c->K, c->T, c->phi[pcur], c->nrm, c->frep, nullptr, 0, c->tiles[pcur],
-                          c->ntiles + pcur, c->nci_blocks, st, nci_aux(c), c->ntiles + pn);
+        return launch_nci(d, c->K, c->phi[pcur], c->nrm, c->frep, nullptr, tile_list(c, pcur), c->nci_blocks,
+                          st, c->aux, c->ntiles + pn, nci_parts);
       }, nci_list_kernels(c)));
       if (rc) return rc;
     }
@@ -335,7 +324,6 @@ int lbm_create(const lbm_params *p, lbm_ctx **out) {
   if (!c) return LBM_ERR_OOM;
   c->P = *p;
   derive_kparams(*p, c->K);
-  build_table(p->dim, p->nci_on ? p->w : 1, c->T);
   c->N = c->K.N;
   c->pop_bytes = store_bytes(*p, c->N);
   cudaError_t e = cudaGetDevice(&c->device);
@@ -354,16 +342,15 @@ int lbm_create(const lbm_params *p, lbm_ctx **out) {
   if (e == cudaSuccess) e = cudaMemset(c->ntiles, 0, 2 * sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&c->lflag, sizeof(int) * 2 * (size_t)ntile);
   if (e == cudaSuccess) e = cudaMemset(c->lflag, 0, sizeof(int) * 2 * (size_t)ntile);
-  if (e == cudaSuccess && p->nci_on && nci_aux_applies(p->dim, c->K)) {
+  if (e == cudaSuccess) e = cudaMalloc(&c->aux.masks, nci_mask_bytes(c->K));
+  if (e == cudaSuccess && p->nci_on && p->dim == 3) {
     e = cudaMalloc(&c->aux.bricks, sizeof(uint4) * nci_brick_count(c->K));
-    if (e == cudaSuccess) e = cudaMalloc(&c->aux.flags, (size_t)ntile);
-    if (e == cudaSuccess) e = cudaMemset(c->aux.flags, 0, (size_t)ntile);
-    if (e == cudaSuccess) e = cudaMalloc(&c->aux.scan_tiles, sizeof(int) * ntile);
+    if (e == cudaSuccess) e = cudaMalloc(&c->aux.scan_units, sizeof(int) * 2 * (size_t)ntile);
     if (e == cudaSuccess) e = cudaMalloc(&c->aux.nscan, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(c->aux.nscan, 0, sizeof(int));
   }
   if (e == cudaSuccess) {
-    c->nci_blocks = nci_list_blocks(p->dim);
+    c->nci_blocks = nci_list_blocks();
     if (c->nci_blocks <= 0) e = cudaErrorInvalidConfiguration;
   }
   if (e == cudaSuccess && p->nci_on && p->store != LBM_STORE_MOMENTS && hydro_split_applies(p->Q, c->K)) {
@@ -415,7 +402,7 @@ void lbm_destroy(lbm_ctx *c) {
   cudaFree(c->diag_part); cudaFree(c->diag_out);
   cudaFree(c->curv_hist); cudaFree(c->curv_part);
   cudaFree(c->tiles[0]); cudaFree(c->tiles[1]); cudaFree(c->ntiles); cudaFree(c->lflag);
-  cudaFree(c->aux.bricks); cudaFree(c->aux.flags); cudaFree(c->aux.scan_tiles); cudaFree(c->aux.nscan);
+  cudaFree(c->aux.masks); cudaFree(c->aux.bricks); cudaFree(c->aux.scan_units); cudaFree(c->aux.nscan);
   delete c;
 }
 
@@ -602,8 +589,8 @@ int lbm_read_nci(lbm_ctx *c, int32_t *partner, double *frep) {
   }
   if ((rc = ensure_stage(c, sizeof(double) * 3 * N))) return rc;
   rc = from_cuda(timed(c, LBM_K_NCI, [&] {
-    return launch_nci(c->P.dim, c->K, c->T, c->phi[c->pcur], c->nrm, c->frep, c->partner, 1, nullptr, nullptr,
-                      c->nci_blocks, c->stream);
+    return launch_nci(c->P.dim, c->K, c->phi[c->pcur], c->nrm, c->frep, c->partner, TileList{}, c->nci_blocks,
+                      c->stream, c->aux);
   }, 2));
   if (rc) return rc;
   if (partner && (rc = d2h(c, partner, c->partner, sizeof(int32_t) * 3 * N))) return rc;
@@ -632,8 +619,8 @@ int lbm_nci_diagnostics(lbm_ctx *c, double *out) {
   }
   // the near-contact pass over the tiles listed for the current phi (the list stays for the next step)
   int rc = from_cuda(timed(c, LBM_K_NCI, [&] {
-    return launch_nci(c->P.dim, c->K, c->T, c->phi[c->pcur], c->nrm, c->frep, nullptr, 0, c->tiles[c->pcur],
-                      c->ntiles + c->pcur, c->nci_blocks, c->stream, nci_aux(c), c->ntiles + (c->pcur ^ 1));
+    return launch_nci(c->P.dim, c->K, c->phi[c->pcur], c->nrm, c->frep, nullptr, tile_list(c, c->pcur),
+                      c->nci_blocks, c->stream, c->aux, c->ntiles + (c->pcur ^ 1));
   }, nci_list_kernels(c)));
   if (rc) return rc;
   rc = from_cuda(timed(c, LBM_K_REDUCE, [&] {

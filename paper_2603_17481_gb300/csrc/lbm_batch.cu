@@ -71,8 +71,8 @@ bool fusable(lbm_ctx *const *ctxs, int n) {
 
 // The near-contact pass of context c on phi[pc] (the list of that buffer), on stream s.
 cudaError_t nci_pass(lbm_ctx *c, int pc, cudaStream_t s) {
-  return launch_nci(c->P.dim, c->K, c->T, c->phi[pc], c->nrm, c->frep, nullptr, 0, c->tiles[pc], c->ntiles + pc,
-                    c->nci_blocks, s, nci_aux(c), c->ntiles + (pc ^ 1));
+  return launch_nci(c->P.dim, c->K, c->phi[pc], c->nrm, c->frep, nullptr, tile_list(c, pc), c->nci_blocks, s,
+                    c->aux, c->ntiles + (pc ^ 1), 1);
 }
 
 // BatchCase of context c for a step from buffer parity (cur, pcur); lists = false leaves the
@@ -188,7 +188,7 @@ int time_dry_step(lbm_batch *b, bool fused, double &ms) {
     const int cur = b->cur0[i], pc = b->pcur0[i];
     if (fused) {
       if (c->P.nci_on) e = nci_pass(c, pc, br);
-    } else if (enqueue_step(c, cur, pc, false, br) != LBM_OK) {
+    } else if (enqueue_step(c, cur, pc, false, br, 1) != LBM_OK) {
       e = cudaErrorUnknown;
     }
   }
@@ -273,7 +273,7 @@ int capture_steps(lbm_batch *b, int g) {
       if (b->fused) {
         if (c->P.nci_on) e = nci_pass(c, b->pcur0[i] ^ q, br);
       } else {
-        rc = enqueue_step(c, b->cur0[i] ^ q, b->pcur0[i] ^ q, true, br);
+        rc = enqueue_step(c, b->cur0[i] ^ q, b->pcur0[i] ^ q, true, br, 1);
       }
     }
     for (size_t s = 0; s < b->branches.size() && e == cudaSuccess; s++) {

@@ -195,16 +195,11 @@ struct KParams {
   float g[3];
   int nci_on, w;
   float A_rep, h0, p, q_th, eta, cos_opp, eps_q, eps_n, eps;
+  float face_t;          // near-contact direction classes: partners of n_a > 0 (a its largest component) have m_a <= face_t
   float Dlap;            // D * 2 / cs^2  (Laplacian link weight factor, Eq. 23 times D)
   float kc;              // kappa / cs^2  (compressive link factor, Eq. 35)
   double rho_g64, drho64;  // the density rule in FP64 for the FP64 momentum integral
 };
-
-// Near-contact window offsets sorted by (|r|^2, canonical index); filled by the host.
-struct NciOffset {
-  int8_t dx, dy, dz, d2;
-};
-constexpr int kMaxOffsets = 342;  // (2*3+1)^3 - 1
 
 // Tile geometry (threads per block = TX*TY*TZ, one cell per thread).
 template <int DIM> struct Tile;
