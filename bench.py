@@ -544,7 +544,7 @@ def run_sweep(args, world, rank, local):
     mlups_single, ms_single_max = whole_job_mlups(world, cells, steps, ms_single, device=f"cuda:{local}")
 
     # the per-case graph (every context's own steps on concurrent branches), the fused batch as is
-    # (one launch per pass over all cases, tile shape 64x4x2 and 4 march rows), and the autotuned
+    # (one launch per pass over all cases, tile shape 32x4x2 and 4 march rows), and the autotuned
     # batch (tile shape and march rows tuned, then the faster of fused and per-case), at each
     # branch count
     results, graph_results, fused_results, configs = {}, {}, {}, {}
@@ -595,7 +595,7 @@ def run_sweep(args, world, rank, local):
                            "what": "CUDA graph of every case's own lbm_step kernels on concurrent branches"},
         "fused_untuned": {"by_branches": {str(ns): round(v[0], 1) for ns, v in fused_results.items()},
                           "what": "one hydrodynamic and one phase-field launch over all cases per step, "
-                                  "64x4x2 tiles, 4 march rows"},
+                                  "32x4x2 tiles, 4 march rows"},
         "tuned_by_branches": {str(ns): round(v[0], 1) for ns, v in results.items()},
         "tuned_config": configs[best],
         "tuned_vs_per_case_graph": round(mlups / max(v[0] for v in graph_results.values()), 3),

@@ -222,7 +222,7 @@ int lbm_batch_create(lbm_ctx *const *ctxs, int n, int nstreams, void *stream, lb
  * one launch of the phase-field pass over all contexts together (persistent grids walking a work
  * list of every case's tiles), with the same per-cell arithmetic as lbm_step, so the results are
  * identical. An autotuner then times, on the contexts' own state and without changing it, the
- * hydrodynamic tile shape (64 x ty x 8/ty cells, ty = 4, 2, 8) and the rows of y per thread of the
+ * hydrodynamic tile shape (32 x ty x 8/ty cells, ty = 4, 2, 8) and the rows of y per thread of the
  * phase-field march (4 or 2), keeps the fastest, and finally times one step of that fused
  * execution against one step of the per-case graph, keeping the fused execution only when it is at
  * least 3 % faster (lbm_batch_config reports both times).

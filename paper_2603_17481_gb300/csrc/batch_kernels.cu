@@ -13,7 +13,7 @@ namespace lbm {
 // current item computes, so an item starts without a chain of dependent global loads, and its
 // parameters are read from shared memory.
 template <class L, int S, int TY>
-__global__ void __launch_bounds__(256, L::Q >= 27 ? 2 : LBM_HYDRO2_MINB)
+__global__ void __launch_bounds__(LX * 8, L::Q >= 27 ? 4 : 6)
 k_hydro2_batch(const BatchCase *__restrict__ cases, const int4 *__restrict__ items, const int nitems) {
   pdl_enter();
   constexpr int TZ = 8 / TY;
@@ -22,7 +22,7 @@ k_hydro2_batch(const BatchCase *__restrict__ cases, const int4 *__restrict__ ite
   __shared__ uint4 s_case[2][WORDS];
   __shared__ int4 s_item[2];
   using T = typename Store<S>::T;
-  const int tid = threadIdx.x + 32 * (threadIdx.y + TY * threadIdx.z);
+  const int tid = threadIdx.x + LX * (threadIdx.y + TY * threadIdx.z);
   auto fetch = [&](int it, int buf) {  // warp 0 copies item it and its case record
     if (tid < 32 && it < nitems) {
       const int4 w = items[it];
@@ -91,9 +91,9 @@ template <class K> int resident(K kernel, int threads) {
 template <class L, int S>
 cudaError_t hydro_batch_ty(int ty, const BatchCase *cases, const int4 *items, int nitems, int blocks, cudaStream_t s) {
   switch (ty) {
-    case 2: return launch_pdl(k_hydro2_batch<L, S, 2>, dim3(blocks), dim3(32, 2, 4), 0, s, cases, items, nitems);
-    case 8: return launch_pdl(k_hydro2_batch<L, S, 8>, dim3(blocks), dim3(32, 8, 1), 0, s, cases, items, nitems);
-    default: return launch_pdl(k_hydro2_batch<L, S, 4>, dim3(blocks), dim3(32, 4, 2), 0, s, cases, items, nitems);
+    case 2: return launch_pdl(k_hydro2_batch<L, S, 2>, dim3(blocks), dim3(LX, 2, 4), 0, s, cases, items, nitems);
+    case 8: return launch_pdl(k_hydro2_batch<L, S, 8>, dim3(blocks), dim3(LX, 8, 1), 0, s, cases, items, nitems);
+    default: return launch_pdl(k_hydro2_batch<L, S, 4>, dim3(blocks), dim3(LX, 4, 2), 0, s, cases, items, nitems);
   }
 }
 template <class L>
@@ -118,7 +118,7 @@ cudaError_t launch_hydro_batch(int Q, int store, int ty, const BatchCase *cases,
 int hydro_batch_blocks(int Q, int store, int ty) {
   // the resident count depends on the lattice (registers), not on the store or the tile shape
   (void)store; (void)ty;
-  return Q == 27 ? resident(k_hydro2_batch<D3Q27, 0, 4>, 256) : resident(k_hydro2_batch<D3Q19, 0, 4>, 256);
+  return Q == 27 ? resident(k_hydro2_batch<D3Q27, 0, 4>, LX * 8) : resident(k_hydro2_batch<D3Q19, 0, 4>, LX * 8);
 }
 
 cudaError_t launch_phase_batch(int rows, const BatchCase *cases, const long long *uoff, int ncases, int blocks,

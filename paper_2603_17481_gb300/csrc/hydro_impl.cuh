@@ -508,10 +508,14 @@ template <> struct Pair<2> {
 };
 
 // The 3D hydrodynamic step with two x-adjacent cells per thread (nx even, Q N <= 2^32). The blocks
-// are 64 x 2 x 2 cells (128 threads), small on purpose: the kernel alternates waiting for memory
+// are 32 x 2 x 4 cells (128 threads), small on purpose: the kernel alternates waiting for memory
 // and computing, so its bandwidth grows with the number of blocks an SM can interleave (six at 80
-// registers; 256 x 128 x 128 D3Q19 FP32 128.5 us, against 142.7 us with three 64 x 4 x 2 blocks of
-// the same registers and this kernel's first form of the loads).
+// registers; 256 x 128 x 128 D3Q19 FP32 127 us, against 142.7 us with three 64 x 4 x 2 blocks of
+// the same registers and this kernel's first form of the loads). A tile is 16 threads wide, so a warp
+// covers two rows: the time goes with the width that the tiles cover, 64 cells wide ones took
+// 55.4 us on 160 x 96 x 96, as much as on 192 x 96 x 96, 32 wide ones take 49.0 (96^3 39.0 -> 31.8, 80^3
+// 27.4 -> 21.4, 144^3 113 -> 97 us, 256 x 128 x 128 131 -> 127). 16 cells wide ones gain 1 to 4 % more on
+// 80, 112 and 144, and lose 5 % on 256 and 17 % on 130 x 120 x 120.
 // For each direction one paired load brings the populations of the source cells x - c_i,
 // x + 1 - c_i when c_x = 0. When c_x = +-1 the pair is shifted by one cell and comes as two single
 // loads: the second one hits the lines of the first in L1, and the thread needs neither its
@@ -524,39 +528,37 @@ template <> struct Pair<2> {
 // index, so the four columns x - 1 .. x + 2 of a stencil row are two 8-byte shared loads. The
 // stencils are evaluated before the pull, which keeps their 36 inputs out of the registers that the
 // populations need.
-// Shared memory of one tile of the paired kernel (the tile is 64 x TY x TZ cells).
+// Threads of a row of a tile, and the shared memory of one tile of the paired kernel (2 LX x TY x TZ cells).
+constexpr int LX = 16;
 template <int TY, int TZ> struct Hydro2Smem {
-  static constexpr int HX = 68, HY = TY + 2, HZ = TZ + 2;  // row pitch 68: column x0 - 1 + j at index j
+  static constexpr int HX = 2 * LX + 4, HY = TY + 2, HZ = TZ + 2;  // column x0 - 1 + j at index j
   static constexpr int NROWS = HY * HZ, FLOATS = NROWS * HX;
 };
 
-// One tile (bx, by, bz) of 64 x TY x TZ cells with a block of 32 x TY x TZ threads. Every thread
+// One tile (bx, by, bz) of 2 LX x TY x TZ cells with a block of LX x TY x TZ threads. Every thread
 // of the block calls it (one barrier inside; a caller looping over tiles adds one between tiles).
-// halves: bit 0 updates the cells x0 .. x0 + 31 (lanes 0 - 15), bit 1 x0 + 32 .. x0 + 63; the
-// lanes of a half that is not updated only help to stage phi.
 template <class L, int S, int MODE, int TY, int TZ>
 __device__ __forceinline__ void hydro2_tile(const KParams &P, const typename Store<S>::T *__restrict__ src,
                                             typename Store<S>::T *__restrict__ dst, const int32_t *__restrict__ phi,
                                             const float4 *__restrict__ frep, float *__restrict__ u_out,
-                                            float *__restrict__ ps_out, const int bx, const int by, const int bz,
-                                            const unsigned halves = 3u) {
+                                            float *__restrict__ ps_out, const int bx, const int by, const int bz) {
   __shared__ __align__(16) float s_phi[Hydro2Smem<TY, TZ>::FLOATS];
   static_assert(L::D == 3, "3D lattices");
   using SL = D3Q27;
   using SM = Hydro2Smem<TY, TZ>;
   constexpr int HX = SM::HX, HY = SM::HY;
-  constexpr int NROWS = SM::NROWS, NWARPS = TY * TZ;
+  constexpr int NROWS = SM::NROWS, NTEAMS = TY * TZ;  // LX threads stage a row
 
   const int lane = threadIdx.x, ty = threadIdx.y, tz = threadIdx.z;
   const int nx = P.nx, ny = P.ny, nz = P.nz;
-  const int x0 = bx * 64, y0 = by * TY, z0 = bz * TZ;
+  const int x0 = bx * 2 * LX, y0 = by * TY, z0 = bz * TZ;
   const int x = x0 + 2 * lane, y = y0 + ty, z = z0 + tz;
-  // stage phi: the pairs (x0 - 2 + 2 lane, x0 - 1 + 2 lane) of each row cover x0 - 2 .. x0 + 61;
-  // lanes 0 and 1 add the pairs at x0 + 62 and x0 + 64 (nx even keeps every pair aligned)
+  // stage phi: the pairs (x0 - 2 + 2 lane, x0 - 1 + 2 lane) of each row cover x0 - 2 .. x0 + 2 LX - 3;
+  // lanes 0 and 1 add the next two pairs (nx even keeps every pair aligned)
   {
     const int xa = wrapn(x0 - 2 + 2 * lane, nx);
-    const int xb = wrapn(x0 + 62 + 2 * lane, nx);
-    for (int r = ty + TY * tz; r < NROWS; r += NWARPS) {
+    const int xb = wrapn(x0 + 2 * LX - 2 + 2 * lane, nx);
+    for (int r = ty + TY * tz; r < NROWS; r += NTEAMS) {
       const int ry = r % HY, rz = r / HY;
       const int Y = wrapn(y0 + ry - 1, ny);
       const int Z = wrapn(z0 + rz - 1, nz);
@@ -567,14 +569,14 @@ __device__ __forceinline__ void hydro2_tile(const KParams &P, const typename Sto
       sr[2 * lane] = phi_of(a.y);
       if (lane < 2) {
         const int2 b = *reinterpret_cast<const int2 *>(row + xb);
-        sr[63 + 2 * lane] = phi_of(b.x);
-        sr[64 + 2 * lane] = phi_of(b.y);
+        sr[2 * LX - 1 + 2 * lane] = phi_of(b.x);
+        sr[2 * LX + 2 * lane] = phi_of(b.y);
       }
     }
   }
   __syncthreads();
   // nx even: x + 1 < nx too; no barrier or shuffle follows
-  if (x >= nx || y >= ny || z >= nz || !((halves >> (lane >> 4)) & 1u)) return;
+  if (x >= nx || y >= ny || z >= nz) return;
 
   // isotropic gradient and Laplacian of phi (Eqs. 22-23) at both cells: columns x - 1 .. x + 2 of
   // the nine stencil rows as two 8-byte shared loads each
@@ -662,17 +664,6 @@ __device__ __forceinline__ void hydro2_tile(const KParams &P, const typename Sto
   if constexpr (MODE == kMoments) *reinterpret_cast<float2 *>(ps_out + idx) = pso.v;
 }
 
-// The near-contact tiles (32 x 8 x 4) holding the two halves of the paired tile (bx, by, bz) of
-// 64 x 2 x 2 cells: tiles 2 bx and 2 bx + 1 of the row (by / 4, bz / 2); the second is -1 beyond
-// the grid.
-static_assert(NciTile<3>::X == 32 && NciTile<3>::Y == 8 && NciTile<3>::Z == 4,
-              "a near-contact tile holds 4 x 2 paired tiles of 64 x 2 x 2 cells in y, z, and half of one in x");
-__device__ __forceinline__ int2 nci_tiles_of_pair(const KParams &P, int bx, int by, int bz) {
-  const int gtx = (P.nx + 31) >> 5, gty = (P.ny + 7) >> 3;
-  const int t0 = 2 * bx + gtx * ((by >> 2) + gty * (bz >> 1));
-  return make_int2(t0, 2 * bx + 1 < gtx ? t0 + 1 : -1);
-}
-
 // (c_y + 1) + 4 (c_z + 1) of directions 16 w .. 16 w + 15, four bits each
 template <class L> constexpr unsigned long long row_codes(int w) {
   unsigned long long m = 0;
@@ -681,43 +672,54 @@ template <class L> constexpr unsigned long long row_codes(int w) {
   return m;
 }
 
-// Asks L2 for the source rows of the populations that tile (bx, by, bz) of 64 x TY x TZ cells will
-// pull: warp (ty, tz) takes its row, lane i direction i (the cells x0 .. x0 + 63 of the row of
+// Asks L2 for the source rows of the populations that tile (bx, by, bz) of 2 LX x TY x TZ cells will
+// pull: a warp takes a row at a time, lane i direction i (the cells x0 .. x0 + 2 LX - 1 of the row of
 // x - c_i; the one cell of a shifted pair outside them lies in a neighbouring tile's lines). A
 // prefetch is a hint: it reads nothing into registers and cannot fault on these in-buffer rows.
 template <class L, int S, int TY, int TZ>
 __device__ __forceinline__ void hydro2_prefetch(const KParams &P, const typename Store<S>::T *src, int bx, int by,
                                                 int bz) {
   using T = typename Store<S>::T;
-  const int i = threadIdx.x;
-  const int y = by * TY + threadIdx.y, z = bz * TZ + threadIdx.z, x0 = bx * 64;
-  if (i >= L::Q || y >= P.ny || z >= P.nz) return;
+  const int tid = threadIdx.x + LX * (threadIdx.y + TY * threadIdx.z), i = tid & 31, x0 = bx * 2 * LX;
+  if (i >= L::Q || x0 >= P.nx) return;
   constexpr unsigned long long c0 = row_codes<L>(0), c1 = row_codes<L>(1);
   const int code = (int)((i < 16 ? c0 >> (4 * i) : c1 >> (4 * (i - 16))) & 15ull);
-  const int Y = wrapn(y - ((code & 3) - 1), P.ny), Z = wrapn(z - ((code >> 2) - 1), P.nz);
-  const T *row = src + ((unsigned)i * (unsigned)P.N + (unsigned)(P.nx * (Y + P.ny * Z) + x0));
-  asm volatile("prefetch.global.L2 [%0];" ::"l"(row));
-  constexpr int PER_LINE = 128 / (int)sizeof(T);
-  if (PER_LINE < 64 && x0 + PER_LINE < P.nx) asm volatile("prefetch.global.L2 [%0];" ::"l"(row + PER_LINE));
+#pragma unroll
+  for (int r = 0; r < TY * TZ; r += LX * TY * TZ / 32) {
+    const int row = r + (tid >> 5), y = by * TY + row % TY, z = bz * TZ + row / TY;
+    if (y >= P.ny || z >= P.nz) continue;
+    const int Y = wrapn(y - ((code & 3) - 1), P.ny), Z = wrapn(z - ((code >> 2) - 1), P.nz);
+    const T *p = src + ((unsigned)i * (unsigned)P.N + (unsigned)(P.nx * (Y + P.ny * Z) + x0));
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+    constexpr int PER_LINE = 128 / (int)sizeof(T);
+    if (PER_LINE < 2 * LX && x0 + PER_LINE < P.nx) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + PER_LINE));
+  }
 }
 
 // Tile of the paired kernel in y and z, and the blocks per SM its registers are sized for: D3Q19 six
 // (80 registers; seven at 72 spill and take 130.6 us against 127.0 in FP32, 110.8 against 114.0 in
 // FP16), D3Q27 five (96 registers, 70.7 us on 160 x 96 x 96 against 77.5 with four at 126).
 struct HydroTile {
-  static constexpr int Y = 2, Z = 2;
+  static constexpr int Y = 2, Z = 4;
 };
+constexpr int kHydro2Threads = LX * HydroTile::Y * HydroTile::Z;
 template <class L, int S> __host__ __device__ constexpr int hydro2_minb() { return L::Q >= 27 ? 5 : (S == 0 ? 6 : 7); }
+// The near-contact tile that holds the paired tile (bx, by, bz) of 32 x 2 x 4 cells.
+static_assert(NciTile<3>::X == 2 * LX && NciTile<3>::Y == 4 * HydroTile::Y && NciTile<3>::Z == HydroTile::Z,
+              "a near-contact tile holds four paired tiles, side by side in y");
+__device__ __forceinline__ int nci_tile_of(const KParams &P, int bx, int by, int bz) {
+  return bx + ((P.nx + 31) >> 5) * ((by >> 2) + ((P.ny + 7) >> 3) * bz);
+}
 // The blocks that ask L2 for their rows: about the first resident wave of a 152-SM GB300.
 constexpr unsigned kPrefetchBlocks = 912;
 
-// listed == nullptr: every cell. Otherwise the split step's first part: only the halves whose
-// near-contact tile is not listed (a block with both halves listed returns at once).
+// listed == nullptr: every cell. Otherwise the split step's first part: only the tiles whose
+// near-contact tile is not listed.
 // The first blocks of the grid, which may be resident while the previous kernel still runs, ask L2
 // for their population rows before they wait for it (128.5 -> 127.0 us on 256 x 128 x 128; asked by
 // every block it cost 384^3 6 %: 1785 us against 1682).
 template <class L, int S, int MODE>
-__global__ void __launch_bounds__(32 * HydroTile::Y * HydroTile::Z, hydro2_minb<L, S>())
+__global__ void __launch_bounds__(kHydro2Threads, hydro2_minb<L, S>())
 k_hydro2(const KParams P, const typename Store<S>::T *__restrict__ src, typename Store<S>::T *__restrict__ dst,
          const int32_t *__restrict__ phi, const float4 *__restrict__ frep, float *__restrict__ u_out,
          float *__restrict__ ps_out, const int *__restrict__ listed, const int by0) {
@@ -728,36 +730,26 @@ k_hydro2(const KParams P, const typename Store<S>::T *__restrict__ src, typename
   if (blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z) < kPrefetchBlocks)
     hydro2_prefetch<L, S, TY, TZ>(P, src, bx, by, bz);
   pdl_enter();
-  unsigned halves = 3u;
-  if (listed) {
-    const int2 t = nci_tiles_of_pair(P, bx, by, bz);
-    halves = (listed[t.x] ? 0u : 1u) | (t.y >= 0 && listed[t.y] ? 0u : 2u);
-    if (halves == 0u) return;  // block-uniform
-  }
-  hydro2_tile<L, S, MODE, TY, TZ>(P, src, dst, phi, frep, u_out, ps_out, bx, by, bz, halves);
+  if (listed && listed[nci_tile_of(P, bx, by, bz)]) return;  // block-uniform
+  hydro2_tile<L, S, MODE, TY, TZ>(P, src, dst, phi, frep, u_out, ps_out, bx, by, bz);
 }
 
-// The split step's second part: the cells of the listed near-contact tiles. Item i of 8 n covers
-// the paired tile (tx / 2, 4 ty + (i & 3), 2 tz + (i >> 2 & 1)) of listed tile i / 8 = (tx, ty, tz);
-// when both near-contact tiles of a pair are listed, the even one's items update both halves and
-// the odd one's items are skipped, so every cell is written once.
+// The split step's second part: the cells of the listed near-contact tiles. Item i of 4 n covers the paired
+// tile (tx, 4 ty + (i & 3), tz) of listed tile i / 4 = (tx, ty, tz).
 template <class L, int S>
-__global__ void __launch_bounds__(32 * HydroTile::Y * HydroTile::Z, hydro2_minb<L, S>())
+__global__ void __launch_bounds__(kHydro2Threads, hydro2_minb<L, S>())
 k_hydro2_listed(const KParams P, const typename Store<S>::T *__restrict__ src, typename Store<S>::T *__restrict__ dst,
                 const int32_t *__restrict__ phi, const float4 *__restrict__ frep, float *__restrict__ u_out,
-                const int *__restrict__ tiles, const int *__restrict__ ntiles, const int *__restrict__ listed) {
+                const int *__restrict__ tiles, const int *__restrict__ ntiles) {
   pdl_enter();
-  const int n8 = 8 * *ntiles;
+  const int n4 = 4 * *ntiles;
   const int gtx = (P.nx + 31) >> 5, gty = (P.ny + 7) >> 3;
-  for (int it = blockIdx.x; it < n8; it += gridDim.x) {
-    const int tile = tiles[it >> 3];
+  for (int it = blockIdx.x; it < n4; it += gridDim.x) {
+    const int tile = tiles[it >> 2];
     const int tx = tile % gtx, tyz = tile / gtx;
-    const int ty = tyz % gty, tz = tyz / gty;
-    if ((tx & 1) && listed[tile - 1]) continue;  // block-uniform: the even tile's items cover it
-    const int bx = tx >> 1, by = 4 * ty + (it & 3), bz = 2 * tz + ((it >> 2) & 1);
-    if (HydroTile::Y * by >= P.ny || HydroTile::Z * bz >= P.nz) continue;
-    const unsigned halves = (tx & 1) ? 2u : (1u | (tx + 1 < gtx && listed[tile + 1] ? 2u : 0u));
-    hydro2_tile<L, S, kStep, HydroTile::Y, HydroTile::Z>(P, src, dst, phi, frep, u_out, nullptr, bx, by, bz, halves);
+    const int ty = tyz % gty, tz = tyz / gty, by = 4 * ty + (it & 3);
+    if (HydroTile::Y * by >= P.ny) continue;
+    hydro2_tile<L, S, kStep, HydroTile::Y, HydroTile::Z>(P, src, dst, phi, frep, u_out, nullptr, tx, by, tz);
     __syncthreads();  // the staged phi of this item is no longer read
   }
 }
@@ -770,8 +762,8 @@ cudaError_t launch_hydro2(const KParams &P, const typename Store<S>::T *src, typ
   const int gy = (P.ny + HydroTile::Y - 1) / HydroTile::Y, gz = (P.nz + HydroTile::Z - 1) / HydroTile::Z;
   cudaError_t e = cudaSuccess;
   for (int by0 = 0; by0 < gy && e == cudaSuccess; by0 += 65535)
-    e = launch_pdl(k_hydro2<L, S, MODE>, dim3((P.nx + 63) / 64, gy - by0 < 65535 ? gy - by0 : 65535, gz),
-                   dim3(32, HydroTile::Y, HydroTile::Z), 0, s, P, src, dst, phi, frep, u, pstar, listed, by0);
+    e = launch_pdl(k_hydro2<L, S, MODE>, dim3((P.nx + 2 * LX - 1) / (2 * LX), gy - by0 < 65535 ? gy - by0 : 65535, gz),
+                   dim3(LX, HydroTile::Y, HydroTile::Z), 0, s, P, src, dst, phi, frep, u, pstar, listed, by0);
   return e;
 }
 
@@ -819,9 +811,8 @@ cudaError_t launch_split_t(int part, const KParams &P, const void *src, void *ds
   const T *a = (const T *)src;
   T *b = (T *)dst;
   if (part == 0) return launch_hydro2<L, S, kStep>(P, a, b, phi, frep, u, nullptr, listed.mark, s);
-  return launch_pdl(k_hydro2_listed<L, S>, dim3(blocks > 0 ? 2 * blocks : 1), dim3(32, HydroTile::Y, HydroTile::Z), 0, s,
-                    P, a, b, phi, frep, u, (const int *)listed.tiles, (const int *)listed.count,
-                    (const int *)listed.mark);
+  return launch_pdl(k_hydro2_listed<L, S>, dim3(blocks > 0 ? 2 * blocks : 1), dim3(LX, HydroTile::Y, HydroTile::Z), 0, s,
+                    P, a, b, phi, frep, u, (const int *)listed.tiles, (const int *)listed.count);
 }
 
 template <class L>

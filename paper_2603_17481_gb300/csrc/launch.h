@@ -70,13 +70,8 @@ cudaError_t phase_prepare(int dim);
 cudaError_t launch_hydro(int Q, int store, int mode, const KParams &P, const void *src, void *dst,
                          const int32_t *phi, const float4 *frep, float *u, float *pstar, cudaStream_t s);
 
-// Resident k_hydro2_batch blocks (256 threads) per SM its registers are sized for (D3Q19; D3Q27 takes 2).
-#ifndef LBM_HYDRO2_MINB
-#define LBM_HYDRO2_MINB 3
-#endif
-
 // The hydrodynamic step split in two launches around the near-contact pass (3D, nx even,
-// Q N <= 2^32: the paired kernel). part 0 updates every 64 x 2 x 2 tile half whose near-contact
+// Q N <= 2^32: the paired kernel). part 0 updates every 32 x 2 x 4 tile whose near-contact
 // tile is not marked in `listed` (those cells are not gated, so they never read frep, and it may
 // run while the near-contact pass writes frep); part 1 walks the listed tiles on 2 `blocks`
 // resident blocks and updates the rest, after the near-contact pass. Each cell is written by
@@ -122,7 +117,7 @@ struct __align__(16) BatchCase {
   TileList prev;        // near-contact list of phi^n, whose marks the phase pass clears
   int ncx;              // x segments of the phase march
 };
-// The paired hydrodynamic kernel over a list of (case, bx, by, bz) tile items of 64 x ty x tz cells
+// The paired hydrodynamic kernel over a list of (case, bx, by, bz) tile items of 32 x ty x tz cells
 // (ty x tz = 8; all cases D3Q19 or D3Q27 per Q, one store type, nx even, Q N <= 2^32), on a grid of
 // `blocks` resident blocks walking the list.
 cudaError_t launch_hydro_batch(int Q, int store, int ty, const BatchCase *cases, const int4 *items, int nitems,

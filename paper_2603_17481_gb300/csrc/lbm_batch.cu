@@ -10,7 +10,7 @@
 //     walking a work list that concatenates every case (batch_kernels.cu);
 //   per-case mode (otherwise, or on request): every context's step on concurrent branches.
 // When the batch can fuse, an autotuner picks, on the batch itself, the hydrodynamic tile shape
-// (64 x ty x tz cells, ty in {4, 2, 8}) and the rows of y per thread of the phase march (4 or 2)
+// (32 x ty x tz cells, ty in {4, 2, 8}) and the rows of y per thread of the phase march (4 or 2)
 // by timing each candidate pass over the whole batch, then times one step of the tuned fused
 // execution against one step of the per-case graph and keeps the faster. Everything it times
 // writes only the next-step buffers and per-step scratch (near-contact list updates off), so the
@@ -107,7 +107,7 @@ int upload_cases(lbm_batch *b) {
   return from_cuda_b(cudaMemcpy(b->d_cases, h.data(), sizeof(BatchCase) * h.size(), cudaMemcpyHostToDevice));
 }
 
-// (case, bx, by, bz) items of the hydrodynamic pass for tiles of 64 x ty x (8 / ty) cells
+// (case, bx, by, bz) items of the hydrodynamic pass for tiles of 32 x ty x (8 / ty) cells
 int upload_items(lbm_batch *b, int ty) {
   std::vector<int4> items;
   const int tz = 8 / ty;
@@ -115,7 +115,7 @@ int upload_items(lbm_batch *b, int ty) {
     const lbm_params &p = b->ctxs[i]->P;
     for (int bz = 0; bz < (p.nz + tz - 1) / tz; bz++)
       for (int by = 0; by < (p.ny + ty - 1) / ty; by++)
-        for (int bx = 0; bx < (p.nx + 63) / 64; bx++) items.push_back(make_int4(i, bx, by, bz));
+        for (int bx = 0; bx < (p.nx + 31) / 32; bx++) items.push_back(make_int4(i, bx, by, bz));
   }
   b->nitems = (int)items.size();
   return from_cuda_b(cudaMemcpy(b->d_items, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice));
@@ -127,7 +127,7 @@ size_t max_items(lbm_batch *b) {
     size_t s = 0;
     for (lbm_ctx *c : b->ctxs) {
       const lbm_params &p = c->P;
-      s += (size_t)((p.nx + 63) / 64) * ((p.ny + ty - 1) / ty) * ((p.nz + 8 / ty - 1) / (8 / ty));
+      s += (size_t)((p.nx + 31) / 32) * ((p.ny + ty - 1) / ty) * ((p.nz + 8 / ty - 1) / (8 / ty));
     }
     m = std::max(m, s);
   }
