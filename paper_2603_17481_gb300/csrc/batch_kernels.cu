@@ -45,14 +45,14 @@ k_hydro2_batch(const BatchCase *__restrict__ cases, const int4 *__restrict__ ite
 }
 
 template <int M>
-__global__ void __launch_bounds__(March3::NT, LBM_MARCH_MINB)
+__global__ void __launch_bounds__(March3::NT, march_minb<M>())
 k_phase3m_batch(const BatchCase *__restrict__ cases, const long long *__restrict__ uoff, const int ncases) {
   pdl_enter();
   // the marks of the lists of phi^n: block b clears those of cases b, b + grid, ...
   for (int c = blockIdx.x; c < ncases; c += gridDim.x) clear_marks(cases[c].prev, threadIdx.x, March3::NT);
   const long long units = uoff[ncases];
   const long long nwarps = (long long)gridDim.x * March3::WARPS;
-  const long long wid = (long long)blockIdx.x * March3::WARPS + (threadIdx.x >> 5);
+  const long long wid = (long long)blockIdx.x * March3::WARPS + __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);
   long long ub = units * wid / nwarps;
   const long long ue = units * (wid + 1) / nwarps;
   if (ub >= ue) return;

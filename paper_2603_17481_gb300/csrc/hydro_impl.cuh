@@ -461,14 +461,6 @@ k_hydro(const KParams P, const typename Store<S>::T *__restrict__ src, typename 
   if (DIM == 3) u_out[2 * NO + (Off)idx] = u2;
 }
 
-// An element at a 32-bit byte offset from a base that is the same for the whole warp.
-template <class T> __device__ __forceinline__ const T *at(const T *base, unsigned bytes) {
-  return reinterpret_cast<const T *>(reinterpret_cast<const char *>(base) + bytes);
-}
-template <class T> __device__ __forceinline__ T *at(T *base, unsigned bytes) {
-  return reinterpret_cast<T *>(reinterpret_cast<char *>(base) + bytes);
-}
-
 // Paired storage access: the populations of two x-adjacent cells as one 8-byte (FP32) or 4-byte
 // (FP16 / BF16) load (ld, x even) or as two single loads (ld2, from any two places), and their
 // store, converted to FP32 as f (loads take w_i, as Store::ld).

@@ -252,42 +252,50 @@ static cudaError_t launch_phase_dim(const KParams &P, const int32_t *phi, const 
 
 // Records once, at context creation, how many k_phase3m blocks the device holds at once (SMs x
 // resident blocks), so that the launches make no non-stream CUDA call (they may be captured).
-static int g_march_slots = 0;
-#ifndef LBM_MARCH_ROWS
-#define LBM_MARCH_ROWS 4
-#endif
-constexpr int kMarchRows = LBM_MARCH_ROWS;  // rows in y per thread of k_phase3m (2 or 4)
+static int g_march_slots2 = 0, g_march_slots4 = 0;  // two and four rows of y per thread
 
 cudaError_t phase_prepare(int dim) {
   static bool done = false;
   if (dim != 3 || done) return cudaSuccess;
-  int dev = 0, sms = 0, perm = 0;
+  int dev = 0, sms = 0, per2 = 0, per4 = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&perm, k_phase3m<kMarchRows>, March3::NT, 0);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per2, k_phase3m<2>, March3::NT, 0);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per4, k_phase3m<4>, March3::NT, 0);
   if (e == cudaSuccess) {
-    g_march_slots = sms * (perm > 0 ? perm : 1);
+    g_march_slots2 = sms * (per2 > 0 ? per2 : 1);
+    g_march_slots4 = sms * (per4 > 0 ? per4 : 1);
     done = true;
   }
   return e;
 }
 
-static cudaError_t launch_phase3(const KParams &P, const int32_t *phi, const float *u, int32_t *phi_out,
-                                 const TileList &next, const TileList &prev, cudaStream_t s) {
-  const cudaError_t e = phase_prepare(3);
-  if (e != cudaSuccess) return e;
-  // one resident wave of warps sharing the (column, plane) units equally, at least MIN_RUN planes each
-  constexpr int M = kMarchRows;
+// One resident wave of warps sharing the (column, plane) units equally, at least MIN_RUN planes each.
+template <int M>
+static cudaError_t launch_march(const KParams &P, const int32_t *phi, const float *u, int32_t *phi_out,
+                                const TileList &next, const TileList &prev, int slots, cudaStream_t s) {
   const int ncx = (P.nx + March3::OUT - 1) / March3::OUT, ncy = (P.ny + M - 1) / M;
   const long long units = (long long)ncx * ncy * P.nz;
   const long long want = (units + March3::MIN_RUN - 1) / March3::MIN_RUN;
   long long blocks = (want + March3::WARPS - 1) / March3::WARPS;
-  if (blocks > g_march_slots) blocks = g_march_slots;
+  if (blocks > slots) blocks = slots;
   if (blocks < 1) blocks = 1;
   const TileList none{};
   return launch_pdl(k_phase3m<M>, dim3((unsigned)blocks), dim3(March3::NT), 0, s, P, phi, u, phi_out,
                     next.tiles ? next : none, next.tiles ? prev : none, ncx, units);
+}
+
+// Two rows per thread up to 44 planes per warp of the four-row kernel, four beyond. A whole step with
+// four and with two: 64^3 40.0 and 36.5 us, 96^3 66.8 and 64.2, 128^3 117.8 and 115.3, 256 x 128 x 128 (34 planes)
+// 210.8 and 207.7, 192^3 (53 planes) 348.5 and 349.2, 256^3 798 and 805, 384^3 2717 and 2754.
+static cudaError_t launch_phase3(const KParams &P, const int32_t *phi, const float *u, int32_t *phi_out,
+                                 const TileList &next, const TileList &prev, cudaStream_t s) {
+  const cudaError_t e = phase_prepare(3);
+  if (e != cudaSuccess) return e;
+  const long long units4 = (long long)((P.nx + March3::OUT - 1) / March3::OUT) * ((P.ny + 3) / 4) * P.nz;
+  if (units4 <= 44LL * March3::WARPS * g_march_slots4)
+    return launch_march<2>(P, phi, u, phi_out, next, prev, g_march_slots2, s);
+  return launch_march<4>(P, phi, u, phi_out, next, prev, g_march_slots4, s);
 }
 
 cudaError_t launch_phase(int dim, const KParams &P, const int32_t *phi, const float *u, int32_t *phi_out,

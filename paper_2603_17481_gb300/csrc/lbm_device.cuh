@@ -179,6 +179,14 @@ __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// An element at a 32-bit byte offset from a base that is the same for the whole warp.
+template <class T> __device__ __forceinline__ const T *at(const T *base, unsigned bytes) {
+  return reinterpret_cast<const T *>(reinterpret_cast<const char *>(base) + bytes);
+}
+template <class T> __device__ __forceinline__ T *at(T *base, unsigned bytes) {
+  return reinterpret_cast<T *>(reinterpret_cast<char *>(base) + bytes);
+}
+
 // Periodic wrap with a fast path for in-range coordinates.
 __device__ __forceinline__ int wrapn(int a, int n) { return (unsigned)a < (unsigned)n ? a : wrapi(a, n); }
 
@@ -195,6 +203,8 @@ struct KParams {
   float g[3];
   int nci_on, w;
   float A_rep, h0, p, q_th, eta, cos_opp, eps_q, eps_n, eps;
+  int32_t gate_lo;       // fixed-point phi outside gate_lo .. gate_lo + gate_span does not pass the interfacial gate
+  uint32_t gate_span;    // (a little wider than the gate, which is taken on binary32 values)
   float face_t;          // near-contact direction classes: partners of n_a > 0 (a its largest component) have m_a <= face_t
   float Dlap;            // D * 2 / cs^2  (Laplacian link weight factor, Eq. 23 times D)
   float kc;              // kappa / cs^2  (compressive link factor, Eq. 35)

@@ -63,14 +63,17 @@ __device__ __forceinline__ float div_ftz(float x, float y) {
 // and odd, so their minmod is the conversion of the integer minmod. One slope and two states per
 // cell and axis, instead of one integer slope per face, took 256 x 128 x 128 from 71.9 to 68.5 us
 // and 384^3 from 825 to 790 us.
-// It is bound by instruction issue and by dependent operations with two warps per scheduler (255
-// registers). Measured and not kept: rows shared by the warps of a block through shared memory (no
+// It is bound by instruction issue and by dependent operations. Four rows per thread run on two warps
+// per scheduler (242 registers), two rows on four (128 registers): two recompute more of their
+// neighbours' rows but wait less, which is the better one where a warp's run is short anyway.
+// The plane's addresses are common to the warp (in uniform registers) and the rows' offsets 32-bit:
+// 256 x 128 x 128 68.7 -> 63.7 us, 384^3 790 -> 743; the gate of the listed tiles is taken on integer bounds
+// first: 63.7 -> 62.2 and 743 -> 729.
+// Measured and not kept: rows shared by the warps of a block through shared memory (no
 // warp recomputes its neighbours' rows of a; the halo warps, the barrier per plane and the spills
-// below 168 registers cost more: 81 - 145 us), two rows per thread at 168 registers (74 us).
+// below 168 registers cost more: 81 - 145 us on 256 x 128 x 128), the loop unrolled by two (64.1).
 // Resident blocks per SM the registers are sized for.
-#ifndef LBM_MARCH_MINB
-#define LBM_MARCH_MINB 2
-#endif
+template <int M> __host__ __device__ constexpr int march_minb() { return M == 2 ? 4 : 2; }
 
 // One warp's march over the planes z0 .. z1 - 1 of the column col (x segment col % ncx, y rows
 // (col / ncx) M ..) of one case.
@@ -98,9 +101,11 @@ __device__ __forceinline__ void march_run(const KParams &P, const int32_t *__res
   const int xs = ix * March3::OUT, ys = iy * M;
   const int x = wrapi(xs + lane - 2, nx);
   const bool xout = lane >= 2 && lane < 2 + March3::OUT && xs + lane - 2 < nx;
-  int yo[NR];  // in-plane offsets of this thread's cells in rows -2 .. M+1
+  // in-plane byte offsets of this thread's cells in rows -2 .. M+1; the plane's address is common to the
+  // warp, so a load or store needs no address arithmetic of its own
+  unsigned yo[NR];
 #pragma unroll
-  for (int i = 0; i < NR; i++) yo[i] = wrapi(ys + i - 2, ny) * nx + x;
+  for (int i = 0; i < NR; i++) yo[i] = 4u * (unsigned)(wrapi(ys + i - 2, ny) * nx + x);
   // near-contact tiles (32 x 8 x 4) touched by the output columns: x tiles tx0 and tx1
   const int tx0 = xs / 32, tx1 = min(xs + March3::OUT - 1, nx - 1) / 32;
   unsigned tflag = 0;  // bit 0: tile tx0, bit 1: tile tx1, for the current group of 4 planes
@@ -128,7 +133,7 @@ __device__ __forceinline__ void march_run(const KParams &P, const int32_t *__res
   int pz = wrapi(z0 - 2, nz) * plane;
   int pz1 = (pz == 0 ? N : pz) - plane, pz2 = (pz1 == 0 ? N : pz1) - plane;
 #pragma unroll
-  for (int i = 0; i < NR; i++) NX[i] = __ldg(phi + pz + yo[i]);
+  for (int i = 0; i < NR; i++) NX[i] = __ldg(at(phi + pz, yo[i]));
 
   for (int p = z0 - 2; p <= z1 + 1; p++) {
     int32_t I2[NR];
@@ -137,18 +142,18 @@ __device__ __forceinline__ void march_run(const KParams &P, const int32_t *__res
     const int pzn = pz + plane == N ? 0 : pz + plane;
     if (p < z1 + 1) {  // phi of the next plane, in flight during this iteration
 #pragma unroll
-      for (int i = 0; i < NR; i++) NX[i] = __ldg(phi + pzn + yo[i]);
+      for (int i = 0; i < NR; i++) NX[i] = __ldg(at(phi + pzn, yo[i]));
     }
     float uzn[M], uxk[M], uyk[NA];
     if (p >= z0) {
 #pragma unroll
-      for (int r = 0; r < M; r++) uzn[r] = __ldg(uz + pz1 + yo[r + 2]);
+      for (int r = 0; r < M; r++) uzn[r] = __ldg(at(uz + pz1, yo[r + 2]));
     }
     if (p >= z0 + 2) {
 #pragma unroll
-      for (int r = 0; r < M; r++) uxk[r] = __ldg(ux + pz2 + yo[r + 2]);
+      for (int r = 0; r < M; r++) uxk[r] = __ldg(at(ux + pz2, yo[r + 2]));
 #pragma unroll
-      for (int i = 0; i < NA; i++) uyk[i] = __ldg(uy + pz2 + yo[i + 1]);
+      for (int i = 0; i < NA; i++) uyk[i] = __ldg(at(uy + pz2, yo[i + 1]));
     }
     // exact differences of the new plane
     float DXp[NR], DYp[NY];
@@ -244,20 +249,27 @@ __device__ __forceinline__ void march_run(const KParams &P, const int32_t *__res
         const float up = uf >= 0.0f ? PY[j] : MY[j + 1];
         TY[j] = __float2int_rn(__fmaf_rn(Dy, YZk[j], __fmaf_rn(k3s_q, __fadd_rn(AY[j], AY[j + 1]), __fmul_rn(uf, up))));
       }
-      bool g0 = false, g1 = false;
+      int32_t vn[M];
+      bool near = false;  // a value that the gate may pass
 #pragma unroll
       for (int r = 0; r < M; r++) {
         const int acc = sh_up_i(TX[r]) - TX[r] + TY[r] - TY[r + 1] + TZk[r] - TZn[r];
+        vn[r] = I0[r + 2] + acc;
         if (xout && ys + r < ny) {
-          const int32_t vn = I0[r + 2] + acc;
-          phi_out[pz2 + yo[r + 2]] = vn;
-          if (tiles && q_gate_value(vn) >= P.q_th) {
-            if ((xs + lane - 2) / 32 == tx0) g0 = true; else g1 = true;
-          }
+          *at(phi_out + pz2, yo[r + 2]) = vn[r];
+          near = near || (unsigned)(vn[r] - P.gate_lo) <= P.gate_span;
         }
       }
       if (tiles) {
-        tflag |= (__any_sync(0xffffffffu, g0) ? 1u : 0u) | (__any_sync(0xffffffffu, g1) ? 2u : 0u);
+        if (__any_sync(0xffffffffu, near)) {
+          bool g0 = false, g1 = false;
+#pragma unroll
+          for (int r = 0; r < M; r++)
+            if (xout && ys + r < ny && q_gate_value(vn[r]) >= P.q_th) {
+              if ((xs + lane - 2) / 32 == tx0) g0 = true; else g1 = true;
+            }
+          tflag |= (__any_sync(0xffffffffu, g0) ? 1u : 0u) | (__any_sync(0xffffffffu, g1) ? 2u : 0u);
+        }
         if ((k & 3) == 3 || k == z1 - 1) {
           if (lane < 2 && ((tflag >> lane) & 1u)) {
             const int tile = (lane ? tx1 : tx0) + gtx * ((ys >> 3) + gty * (k >> 2));
@@ -303,14 +315,15 @@ __device__ __forceinline__ void clear_marks(const TileList &prev, const long lon
 
 // The grid's warps share the (column, plane) units of one case equally.
 template <int M>
-__global__ void __launch_bounds__(March3::NT, LBM_MARCH_MINB)
+__global__ void __launch_bounds__(March3::NT, march_minb<M>())
 k_phase3m(const KParams P, const int32_t *__restrict__ phi, const float *__restrict__ u,
           int32_t *__restrict__ phi_out, const TileList next, const TileList prev, const int ncx,
           const long long units) {
   pdl_enter();
   clear_marks(prev, (long long)blockIdx.x * March3::NT + threadIdx.x, (long long)gridDim.x * March3::NT);
   const long long nwarps = (long long)gridDim.x * March3::WARPS;
-  const long long wid = (long long)blockIdx.x * March3::WARPS + (threadIdx.x >> 5);
+  // (the shuffle tells the compiler that it is common to the warp)
+  const long long wid = (long long)blockIdx.x * March3::WARPS + __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);
   long long ub = units * wid / nwarps;
   const long long ue = units * (wid + 1) / nwarps;
   const int nz = P.nz;
