@@ -12,6 +12,8 @@ struct ProfPair {
   cudaEvent_t a, b;
 };
 
+constexpr int kListWords = 4;  // words before the marks: the counts of the two lists and of the scan list
+
 struct lbm_ctx {
   lbm_params P;
   lbm::KParams K;
@@ -28,8 +30,9 @@ struct lbm_ctx {
   double *stage = nullptr;
   size_t stage_bytes = 0;
   int32_t *partner = nullptr;
+  char *small = nullptr;  // one allocation of the buffers from here to aux, and of red_part, red_out
   int *tiles[2] = {nullptr, nullptr};
-  int *ntiles = nullptr;  // 2 counters, one per phi buffer
+  int *ntiles = nullptr;  // 2 counters, one per phi buffer (of kListWords, the marks follow them)
   int *lflag = nullptr;   // 2 x ntile marks: tile listed for phi[k]
   int ntile = 0;          // near-contact tiles of the grid
   lbm::NciAux aux;        // near-contact masks, brick ranges and scan lists

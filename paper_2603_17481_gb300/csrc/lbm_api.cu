@@ -213,9 +213,8 @@ T *mapped_view(T *p, size_t bytes, bool write) {
 // rho_bar from the exact phi sum; also records the phi-mass reference of the conservation check
 // and lists the near-contact tiles of the initial phi.
 int finish_init(lbm_ctx *c) {
-  int rc = from_cuda(cudaMemsetAsync(c->ntiles, 0, 2 * sizeof(int), c->stream));
-  if (rc) return rc;
-  rc = from_cuda(cudaMemsetAsync(c->lflag, 0, sizeof(int) * 2 * (size_t)c->ntile, c->stream));
+  // the counts and, behind them, the marks
+  int rc = from_cuda(cudaMemsetAsync(c->ntiles, 0, sizeof(int) * (kListWords + 2 * (size_t)c->ntile), c->stream));
   if (rc) return rc;
   rc = from_cuda(launch_gate_tiles(c->P.dim, c->K, c->phi[c->pcur], tile_list(c, c->pcur), c->stream));
   if (rc) return rc;
@@ -340,18 +339,33 @@ int lbm_create(const lbm_params *p, lbm_ctx **out) {
   if (e == cudaSuccess) e = cudaMalloc(&c->nrm, sizeof(float4) * c->N);
   const int ntile = tile_count(p->dim, c->K);
   c->ntile = ntile;
-  if (e == cudaSuccess) e = cudaMalloc(&c->tiles[0], sizeof(int) * ntile);
-  if (e == cudaSuccess) e = cudaMalloc(&c->tiles[1], sizeof(int) * ntile);
-  if (e == cudaSuccess) e = cudaMalloc(&c->ntiles, 2 * sizeof(int));
-  if (e == cudaSuccess) e = cudaMemset(c->ntiles, 0, 2 * sizeof(int));
-  if (e == cudaSuccess) e = cudaMalloc(&c->lflag, sizeof(int) * 2 * (size_t)ntile);
-  if (e == cudaSuccess) e = cudaMemset(c->lflag, 0, sizeof(int) * 2 * (size_t)ntile);
-  if (e == cudaSuccess) e = cudaMalloc(&c->aux.masks, nci_mask_bytes(c->K));
-  if (e == cudaSuccess && p->nci_on && p->dim == 3) {
-    e = cudaMalloc(&c->aux.bricks, sizeof(uint4) * nci_brick_count(c->K));
-    if (e == cudaSuccess) e = cudaMalloc(&c->aux.scan_units, sizeof(int) * 2 * (size_t)ntile);
-    if (e == cudaSuccess) e = cudaMalloc(&c->aux.nscan, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(c->aux.nscan, 0, sizeof(int));
+  // the small buffers share one allocation (each would cost the creation some 100 us): first the
+  // counters and marks, which start at zero, then lists, bricks, masks and reduction results
+  const bool bricks = p->nci_on && p->dim == 3;
+  size_t bytes = 0;
+  auto place = [&](size_t n) {
+    const size_t at = bytes;
+    bytes += (n + 255) / 256 * 256;
+    return at;
+  };
+  const size_t zero = sizeof(int) * (kListWords + 2 * (size_t)ntile), o_zero = place(zero),
+               o_tiles = place(sizeof(int) * 2 * (size_t)ntile),
+               o_units = place(bricks ? sizeof(int) * 2 * (size_t)ntile : 0),
+               o_bricks = place(bricks ? sizeof(uint4) * nci_brick_count(c->K) : 0), o_masks = place(nci_mask_bytes(c->K)),
+               o_red = place(sizeof(ReduceOut) * (kReduceBlocks + 1));
+  if (e == cudaSuccess) e = cudaMalloc(&c->small, bytes);
+  if (e == cudaSuccess) e = cudaMemset(c->small, 0, zero);
+  if (e == cudaSuccess) {
+    c->ntiles = reinterpret_cast<int *>(c->small + o_zero);
+    c->lflag = c->ntiles + kListWords;
+    c->tiles[0] = reinterpret_cast<int *>(c->small + o_tiles);
+    c->tiles[1] = c->tiles[0] + ntile;
+    c->aux.nscan = c->ntiles + 2;
+    c->aux.masks = reinterpret_cast<unsigned *>(c->small + o_masks);
+    c->aux.scan_units = bricks ? reinterpret_cast<int *>(c->small + o_units) : nullptr;
+    c->aux.bricks = bricks ? reinterpret_cast<uint4 *>(c->small + o_bricks) : nullptr;
+    c->red_part = reinterpret_cast<ReduceOut *>(c->small + o_red);
+    c->red_out = c->red_part + kReduceBlocks;
   }
   if (e == cudaSuccess) {
     c->nci_blocks = nci_list_blocks();
@@ -371,8 +385,6 @@ int lbm_create(const lbm_params *p, lbm_ctx **out) {
   // the static scratch of lbm_mass_noalloc is taken here, once per device, while allocating is
   // allowed; a failure is not the context's (lbm_mass_noalloc repeats the look-up and reports it)
   if (e == cudaSuccess) (void)lbm_noalloc_prepare_device();
-  if (e == cudaSuccess) e = cudaMalloc(&c->red_part, sizeof(ReduceOut) * kReduceBlocks);
-  if (e == cudaSuccess) e = cudaMalloc(&c->red_out, sizeof(ReduceOut));
   if (e == cudaSuccess) e = cudaMemset(c->u, 0, sizeof(float) * 3 * c->N);
   if (e == cudaSuccess) e = cudaMemset(c->frep, 0, sizeof(float4) * c->N);
   if (e == cudaSuccess) e = cudaMemset(c->phi[0], 0, sizeof(int32_t) * c->N);
@@ -402,11 +414,9 @@ void lbm_destroy(lbm_ctx *c) {
   cudaFree(c->pop[0]); cudaFree(c->pop[1]);
   cudaFree(c->phi[0]); cudaFree(c->phi[1]);
   cudaFree(c->u); cudaFree(c->frep); cudaFree(c->nrm); cudaFree(c->mom); cudaFree(c->stage);
-  cudaFree(c->partner); cudaFree(c->red_part); cudaFree(c->red_out);
+  cudaFree(c->partner); cudaFree(c->small);
   cudaFree(c->diag_part); cudaFree(c->diag_out);
   cudaFree(c->curv_hist); cudaFree(c->curv_part);
-  cudaFree(c->tiles[0]); cudaFree(c->tiles[1]); cudaFree(c->ntiles); cudaFree(c->lflag);
-  cudaFree(c->aux.masks); cudaFree(c->aux.bricks); cudaFree(c->aux.scan_units); cudaFree(c->aux.nscan);
   delete c;
 }
 
