@@ -136,8 +136,8 @@ int lbm_step(lbm_ctx *ctx, int n);
  * of the context, while the context stream updates the other cells, which are not gated and so do
  * not read F_rep (Eq. 73); the streams join before the phase-field update. Each cell is updated by
  * one of the two launches with the same arithmetic, so every state is bit-identical to the
- * one-stream step's. blocks > 0 runs it with that many resident near-contact scan blocks (capped
- * at one per SM); blocks = 0 (the default) runs every step on the context stream alone. Takes
+ * one-stream step's. blocks > 0 runs it with a near-contact scan over that many SMs' worth of blocks
+ * (capped at the device's SMs); blocks = 0 (the default) runs every step on the context stream alone. Takes
  * effect at the next lbm_step or batch capture. blocks < 0 or NULL ctx: LBM_ERR_ARG; blocks > 0
  * on a context where the split step does not apply: LBM_ERR_STATE. */
 int lbm_set_overlap(lbm_ctx *ctx, int blocks);

@@ -502,8 +502,9 @@ template <> struct Pair<2> {
 // The 3D hydrodynamic step with two x-adjacent cells per thread (nx even, Q N <= 2^32). The blocks
 // are 32 x 2 x 4 cells (128 threads), small on purpose: the kernel alternates waiting for memory
 // and computing, so its bandwidth grows with the number of blocks an SM can interleave (six at 80
-// registers; 256 x 128 x 128 D3Q19 FP32 127 us, against 142.7 us with three 64 x 4 x 2 blocks of
-// the same registers and this kernel's first form of the loads). A tile is 16 threads wide, so a warp
+// registers; 256 x 128 x 128 D3Q19 FP32 128 us, 5.5 TB/s of its 168 B a cell, against 142.7 us with
+// three 64 x 4 x 2 blocks of the same registers and this kernel's first form of the loads; its reads
+// and writes alone, without the physics between them, take 122 us). A tile is 16 threads wide, so a warp
 // covers two rows: the time goes with the width that the tiles cover, 64 cells wide ones took
 // 55.4 us on 160 x 96 x 96, as much as on 192 x 96 x 96, 32 wide ones take 49.0 (96^3 39.0 -> 31.8, 80^3
 // 27.4 -> 21.4, 144^3 113 -> 97 us, 256 x 128 x 128 131 -> 127). 16 cells wide ones gain 1 to 4 % more on
@@ -689,8 +690,9 @@ __device__ __forceinline__ void hydro2_prefetch(const KParams &P, const typename
 }
 
 // Tile of the paired kernel in y and z, and the blocks per SM its registers are sized for: D3Q19 six
-// (80 registers; seven at 72 spill and take 130.6 us against 127.0 in FP32, 110.8 against 114.0 in
-// FP16), D3Q27 five (96 registers, 70.7 us on 160 x 96 x 96 against 77.5 with four at 126).
+// in FP32 (80 registers: 128.2 us on 256 x 128 x 128; seven at 72 spill: 135.0, five 148.5) and seven
+// with 2-byte stores (107.9; six 109.5, eight 120.9), D3Q27 five (96 registers: 64.2 us on
+// 160 x 96 x 96; six 71.7, four 69.6).
 struct HydroTile {
   static constexpr int Y = 2, Z = 4;
 };
@@ -709,7 +711,7 @@ constexpr unsigned kPrefetchBlocks = 912;
 // near-contact tile is not listed.
 // The first blocks of the grid, which may be resident while the previous kernel still runs, ask L2
 // for their population rows before they wait for it (128.5 -> 127.0 us on 256 x 128 x 128; asked by
-// every block it cost 384^3 6 %: 1785 us against 1682).
+// every block it cost 384^3 6 %: 1785 us against 1682; both with tiles of 64 x 2 x 2 cells).
 template <class L, int S, int MODE>
 __global__ void __launch_bounds__(kHydro2Threads, hydro2_minb<L, S>())
 k_hydro2(const KParams P, const typename Store<S>::T *__restrict__ src, typename Store<S>::T *__restrict__ dst,

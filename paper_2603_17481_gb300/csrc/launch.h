@@ -98,8 +98,8 @@ struct March3 {
   static constexpr int WARPS = 4;      // warps per block
   static constexpr int NT = 32 * WARPS;
   // fewest planes per warp before the grid is shrunk: a run of n planes takes n + 4 iterations, and
-  // a small grid is bound by the time of one run, not by the work (48^3: 18.5 us with runs of 8,
-  // 11.7 with runs of 2; 128 x 64 x 64: 21.0 and 17.7)
+  // a small grid is bound by the time of one run, not by the work (a 48^3 pass: 18.5 us with runs of
+  // 8, 10.3 with runs of 2; its whole step 33.6 us with 2, 36.2 with 1, 35.4 with 3)
   static constexpr int MIN_RUN = 2;
 };
 

@@ -9,9 +9,12 @@
 //   nrm      N float4     interface normals, valid at gated cells only
 //   mom      4*N float    u and p* of lbm_read_fields / lbm_mass (allocated on first use)
 //   stage    k*N double   FP64 staging of host I/O (allocated on first use, grown as needed)
-//   tiles[2] int          near-contact tiles holding an interfacial cell of phi[k] (+ 2 counts)
-//   lflag    2 x int      per near-contact tile and phi buffer: the tile is in that buffer's list
-//   red      reduction partials and result
+//   small    one allocation of
+//     ntiles  kListWords int  counts of tiles[0], tiles[1] and of the scan units
+//     lflag   2 x int     per near-contact tile and phi buffer: the tile is in that buffer's list
+//     tiles[2] int        near-contact tiles holding an interfacial cell of phi[k]
+//     aux                 direction masks (N bytes); with nci_on in 3D the scan units and brick ranges
+//     red                 reduction partials and result
 #include <cuda.h>  // driver API types (CUpointer_attribute); no driver symbols are linked
 
 #include <algorithm>
