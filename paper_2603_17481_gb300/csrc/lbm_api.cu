@@ -26,6 +26,7 @@
 #include <vector>
 
 #include "ctx.h"
+#include "gate_bounds.h"
 
 using namespace lbm;
 
@@ -109,10 +110,7 @@ void derive_kparams(const lbm_params &p, KParams &K) {
   K.eps = (float)p.eps;
   K.Dlap = (float)(p.D * 6.0);
   K.kc = (float)(3.0 * 4.0 * p.D / p.eps);
-  // phi (1 - phi) >= q_th between these values of phi (the whole unit interval where q_th is none of the gate's)
-  const double edge = 0.5 * (1.0 - std::sqrt(std::max(0.0, 1.0 - 4.0 * (p.q_th > 0.0 ? p.q_th : 0.0)))) - 1e-5;
-  K.gate_lo = (int32_t)std::floor(edge * 1073741824.0);
-  K.gate_span = (uint32_t)(std::ceil((1.0 - edge) * 1073741824.0) - (double)K.gate_lo);
+  gate_bounds(K.q_th, K.gate_lo, K.gate_span);
   // The largest m_a of a normal m (|m| <= 1) with n.m <= cos_opp < 0, for any n (|n| <= 1) whose largest
   // component is n_a > 0: n.m >= n_a m_a - |n_t| sqrt(1 - m_a^2) with n_a >= |n| / sqrt(3), which is at most
   // cos_opp only if m_a <= sin(psi), -cos(psi + asin(1 / sqrt(3))) = cos_opp (or m_a <= 0 where psi < 0). The

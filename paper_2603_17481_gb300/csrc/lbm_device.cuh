@@ -204,7 +204,7 @@ struct KParams {
   int nci_on, w;
   float A_rep, h0, p, q_th, eta, cos_opp, eps_q, eps_n, eps;
   int32_t gate_lo;       // fixed-point phi outside gate_lo .. gate_lo + gate_span does not pass the interfacial gate
-  uint32_t gate_span;    // (a little wider than the gate, which is taken on binary32 values)
+  uint32_t gate_span;    // (gate_bounds.h)
   float face_t;          // near-contact direction classes: partners of n_a > 0 (a its largest component) have m_a <= face_t
   float Dlap;            // D * 2 / cs^2  (Laplacian link weight factor, Eq. 23 times D)
   float kc;              // kappa / cs^2  (compressive link factor, Eq. 35)

@@ -257,7 +257,7 @@ __device__ __forceinline__ void march_run(const KParams &P, const int32_t *__res
         vn[r] = I0[r + 2] + acc;
         if (xout && ys + r < ny) {
           *at(phi_out + pz2, yo[r + 2]) = vn[r];
-          near = near || (unsigned)(vn[r] - P.gate_lo) <= P.gate_span;
+          near = near || (unsigned)vn[r] - (unsigned)P.gate_lo <= P.gate_span;
         }
       }
       if (tiles) {
