@@ -271,7 +271,7 @@ cudaError_t phase_prepare(int dim) {
 }
 
 // One resident wave of warps sharing the (column, plane) units equally, at least MIN_RUN planes each.
-template <int M>
+template <int M, class Off = unsigned>
 static cudaError_t launch_march(const KParams &P, const int32_t *phi, const float *u, int32_t *phi_out,
                                 const TileList &next, const TileList &prev, int slots, cudaStream_t s) {
   const int ncx = (P.nx + March3::OUT - 1) / March3::OUT, ncy = (P.ny + M - 1) / M;
@@ -281,7 +281,7 @@ static cudaError_t launch_march(const KParams &P, const int32_t *phi, const floa
   if (blocks > slots) blocks = slots;
   if (blocks < 1) blocks = 1;
   const TileList none{};
-  return launch_pdl(k_phase3m<M>, dim3((unsigned)blocks), dim3(March3::NT), 0, s, P, phi, u, phi_out,
+  return launch_pdl(k_phase3m<M, Off>, dim3((unsigned)blocks), dim3(March3::NT), 0, s, P, phi, u, phi_out,
                     next.tiles ? next : none, next.tiles ? prev : none, ncx, units);
 }
 
@@ -292,6 +292,8 @@ static cudaError_t launch_phase3(const KParams &P, const int32_t *phi, const flo
                                  const TileList &next, const TileList &prev, cudaStream_t s) {
   const cudaError_t e = phase_prepare(3);
   if (e != cudaSuccess) return e;
+  if (march_wide(P))
+    return launch_march<4, unsigned long long>(P, phi, u, phi_out, next, prev, g_march_slots4, s);
   const long long units4 = (long long)((P.nx + March3::OUT - 1) / March3::OUT) * ((P.ny + 3) / 4) * P.nz;
   if (units4 <= 44LL * March3::WARPS * g_march_slots4)
     return launch_march<2>(P, phi, u, phi_out, next, prev, g_march_slots2, s);

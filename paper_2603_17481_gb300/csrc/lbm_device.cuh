@@ -179,11 +179,11 @@ __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// An element at a 32-bit byte offset from a base that is the same for the whole warp.
-template <class T> __device__ __forceinline__ const T *at(const T *base, unsigned bytes) {
+// An element at a byte offset (32-bit unless stated) from a base that is the same for the whole warp.
+template <class T, class Off> __device__ __forceinline__ const T *at(const T *base, Off bytes) {
   return reinterpret_cast<const T *>(reinterpret_cast<const char *>(base) + bytes);
 }
-template <class T> __device__ __forceinline__ T *at(T *base, unsigned bytes) {
+template <class T, class Off> __device__ __forceinline__ T *at(T *base, Off bytes) {
   return reinterpret_cast<T *>(reinterpret_cast<char *>(base) + bytes);
 }
 

@@ -76,8 +76,8 @@ __device__ __forceinline__ float div_ftz(float x, float y) {
 template <int M> __host__ __device__ constexpr int march_minb() { return M == 2 ? 4 : 2; }
 
 // One warp's march over the planes z0 .. z1 - 1 of the column col (x segment col % ncx, y rows
-// (col / ncx) M ..) of one case.
-template <int M>
+// (col / ncx) M ..) of one case. Off: the type of a row's byte offset within its plane (march_wide).
+template <int M, class Off = unsigned>
 __device__ __forceinline__ void march_run(const KParams &P, const int32_t *__restrict__ phi, const float *__restrict__ u,
                                           int32_t *__restrict__ phi_out, int *__restrict__ tiles,
                                           int *__restrict__ ntiles, int *__restrict__ lflag, const int ncx,
@@ -103,9 +103,9 @@ __device__ __forceinline__ void march_run(const KParams &P, const int32_t *__res
   const bool xout = lane >= 2 && lane < 2 + March3::OUT && xs + lane - 2 < nx;
   // in-plane byte offsets of this thread's cells in rows -2 .. M+1; the plane's address is common to the
   // warp, so a load or store needs no address arithmetic of its own
-  unsigned yo[NR];
+  Off yo[NR];
 #pragma unroll
-  for (int i = 0; i < NR; i++) yo[i] = 4u * (unsigned)(wrapi(ys + i - 2, ny) * nx + x);
+  for (int i = 0; i < NR; i++) yo[i] = (Off)4 * (Off)(wrapi(ys + i - 2, ny) * nx + x);
   // near-contact tiles (32 x 8 x 4) touched by the output columns: x tiles tx0 and tx1
   const int tx0 = xs / 32, tx1 = min(xs + March3::OUT - 1, nx - 1) / 32;
   unsigned tflag = 0;  // bit 0: tile tx0, bit 1: tile tx1, for the current group of 4 planes
@@ -313,8 +313,11 @@ __device__ __forceinline__ void clear_marks(const TileList &prev, const long lon
   for (long long i = rank; i < n; i += threads) prev.mark[prev.tiles[i]] = 0;
 }
 
+// Planes whose byte offsets need more than 32 bits: nx ny > 2^30, which within N < 2^31 means nz = 1.
+inline bool march_wide(const KParams &P) { return (long long)P.nx * P.ny > (1LL << 30); }
+
 // The grid's warps share the (column, plane) units of one case equally.
-template <int M>
+template <int M, class Off = unsigned>
 __global__ void __launch_bounds__(March3::NT, march_minb<M>())
 k_phase3m(const KParams P, const int32_t *__restrict__ phi, const float *__restrict__ u,
           int32_t *__restrict__ phi_out, const TileList next, const TileList prev, const int ncx,
@@ -332,7 +335,7 @@ k_phase3m(const KParams P, const int32_t *__restrict__ phi, const float *__restr
     const int z0 = (int)(ub - col * nz);
     const int z1 = (int)min((long long)nz, (long long)z0 + (ue - ub));
     ub += z1 - z0;
-    march_run<M>(P, phi, u, phi_out, next.tiles, next.count, next.mark, ncx, col, z0, z1);
+    march_run<M, Off>(P, phi, u, phi_out, next.tiles, next.count, next.mark, ncx, col, z0, z1);
   }
 }
 
