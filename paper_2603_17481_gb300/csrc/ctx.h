@@ -30,6 +30,7 @@ struct lbm_ctx {
   double *stage = nullptr;
   size_t stage_bytes = 0;
   int32_t *partner = nullptr;
+  unsigned *read_masks = nullptr;  // masks of lbm_read_nci on a context without the repulsion
   char *small = nullptr;  // one allocation of the buffers from here to aux, and of red_part, red_out
   int *tiles[2] = {nullptr, nullptr};
   int *ntiles = nullptr;  // 2 counters, one per phi buffer (of kListWords, the marks follow them)

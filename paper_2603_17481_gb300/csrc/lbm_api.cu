@@ -13,8 +13,9 @@
 //     ntiles  kListWords int  counts of tiles[0], tiles[1] and of the scan units
 //     lflag   2 x int     per near-contact tile and phi buffer: the tile is in that buffer's list
 //     tiles[2] int        near-contact tiles holding an interfacial cell of phi[k]
-//     aux                 direction masks (N bytes); with nci_on in 3D the scan units and brick ranges
+//     aux                 with nci_on: direction masks (N bytes); in 3D the scan units and brick ranges
 //     red                 reduction partials and result
+//   read_masks N bytes    direction masks of lbm_read_nci with nci_on = 0 (allocated on first use)
 #include <cuda.h>  // driver API types (CUpointer_attribute); no driver symbols are linked
 
 #include <algorithm>
@@ -352,7 +353,8 @@ int lbm_create(const lbm_params *p, lbm_ctx **out) {
   const size_t zero = sizeof(int) * (kListWords + 2 * (size_t)ntile), o_zero = place(zero),
                o_tiles = place(sizeof(int) * 2 * (size_t)ntile),
                o_units = place(bricks ? sizeof(int) * 2 * (size_t)ntile : 0),
-               o_bricks = place(bricks ? sizeof(uint4) * nci_brick_count(c->K) : 0), o_masks = place(nci_mask_bytes(c->K)),
+               o_bricks = place(bricks ? sizeof(uint4) * nci_brick_count(c->K) : 0),
+               o_masks = place(p->nci_on ? nci_mask_bytes(c->K) : 0),
                o_red = place(sizeof(ReduceOut) * (kReduceBlocks + 1));
   if (e == cudaSuccess) e = cudaMalloc(&c->small, bytes);
   if (e == cudaSuccess) e = cudaMemset(c->small, 0, zero);
@@ -362,7 +364,7 @@ int lbm_create(const lbm_params *p, lbm_ctx **out) {
     c->tiles[0] = reinterpret_cast<int *>(c->small + o_tiles);
     c->tiles[1] = c->tiles[0] + ntile;
     c->aux.nscan = c->ntiles + 2;
-    c->aux.masks = reinterpret_cast<unsigned *>(c->small + o_masks);
+    c->aux.masks = p->nci_on ? reinterpret_cast<unsigned *>(c->small + o_masks) : nullptr;
     c->aux.scan_units = bricks ? reinterpret_cast<int *>(c->small + o_units) : nullptr;
     c->aux.bricks = bricks ? reinterpret_cast<uint4 *>(c->small + o_bricks) : nullptr;
     c->red_part = reinterpret_cast<ReduceOut *>(c->small + o_red);
@@ -415,7 +417,7 @@ void lbm_destroy(lbm_ctx *c) {
   cudaFree(c->pop[0]); cudaFree(c->pop[1]);
   cudaFree(c->phi[0]); cudaFree(c->phi[1]);
   cudaFree(c->u); cudaFree(c->frep); cudaFree(c->nrm); cudaFree(c->mom); cudaFree(c->stage);
-  cudaFree(c->partner); cudaFree(c->small);
+  cudaFree(c->partner); cudaFree(c->read_masks); cudaFree(c->small);
   cudaFree(c->diag_part); cudaFree(c->diag_out);
   cudaFree(c->curv_hist); cudaFree(c->curv_part);
   delete c;
@@ -601,6 +603,14 @@ int lbm_read_nci(lbm_ctx *c, int32_t *partner, double *frep) {
       c->partner = nullptr;
       return from_cuda(e);
     }
+  }
+  if (!c->aux.masks) {  // with the repulsion off only this pass needs them
+    cudaError_t e = cudaMalloc(&c->read_masks, nci_mask_bytes(c->K));
+    if (e != cudaSuccess) {
+      c->read_masks = nullptr;
+      return from_cuda(e);
+    }
+    c->aux.masks = c->read_masks;
   }
   if ((rc = ensure_stage(c, sizeof(double) * 3 * N))) return rc;
   rc = from_cuda(timed(c, LBM_K_NCI, [&] {
