@@ -25,13 +25,18 @@
 
 namespace lbm {
 
+// Tile shapes of the near-contact lists (2D: also of the phase kernel).
 template <int DIM> struct PhaseGeom {
   static constexpr int TX = PhaseTile<DIM>::X, TY = PhaseTile<DIM>::Y, TZ = PhaseTile<DIM>::Z;
-  static constexpr int HX = TX + 4, HY = TY + 4, HZ = DIM == 3 ? TZ + 4 : 1;  // phi, halo 2
-  static constexpr int AX = TX + 2, AY = TY + 2, AZ = DIM == 3 ? TZ + 2 : 1;  // a, halo 1
-  static constexpr int NB = HX * HY * HZ, NA = AX * AY * AZ, NT = TX * TY * TZ;
+  static constexpr int NT = TX * TY * TZ;
+};
+// The 2D phase kernel's shared-memory boxes and face transfers.
+struct Phase2 : PhaseGeom<2> {
+  static_assert(TZ == 1, "a plane");
+  static constexpr int HX = TX + 4, HY = TY + 4, NB = HX * HY;  // phi, halo 2
+  static constexpr int AX = TX + 2, AY = TY + 2, NA = AX * AY;  // a, halo 1
   // face transfers: faces of the tile cells on their high side plus the low boundary faces
-  static constexpr int FX = (TX + 1) * TY * TZ, FY = TX * (TY + 1) * TZ, FZ = DIM == 3 ? TX * TY * (TZ + 1) : 0;
+  static constexpr int FX = (TX + 1) * TY, FY = TX * (TY + 1);
 };
 
 __device__ __forceinline__ int32_t minmod_i(int32_t a, int32_t b) {
@@ -42,67 +47,39 @@ __device__ __forceinline__ int32_t minmod_i(int32_t a, int32_t b) {
 
 // Transfer across the face between cells p and p + e_AX (tile-local coordinates, p may be one
 // cell below the tile). s_phi has halo 2, s_a halo 1.
-template <int DIM, int AXIS>
+template <int AXIS>
 __device__ __forceinline__ int32_t face_transfer(const KParams &P, const int32_t *s_phi, const float *s_a,
-                                                 const float *__restrict__ u, int px, int py, int pz,
-                                                 int gx, int gy, int gz) {
-  using G = PhaseGeom<DIM>;
-  constexpr int SX = 1, SY = G::HX, SZ = G::HX * G::HY;         // phi-box strides
-  constexpr int AXS = 1, AYS = G::AX, AZS = G::AX * G::AY;       // a-box strides
-  constexpr int E = AXIS == 0 ? SX : (AXIS == 1 ? SY : SZ);
-  constexpr int EA = AXIS == 0 ? AXS : (AXIS == 1 ? AYS : AZS);
-  const int b = (DIM == 3 ? (pz + 2) * SZ : 0) + (py + 2) * SY + px + 2;
-  const int ba = (DIM == 3 ? (pz + 1) * AZS : 0) + (py + 1) * AYS + px + 1;
+                                                 const float *__restrict__ u, int px, int py, int gx, int gy) {
+  using G = Phase2;
+  constexpr int SX = 1, SY = G::HX;    // phi-box strides
+  constexpr int AXS = 1, AYS = G::AX;  // a-box strides
+  constexpr int E = AXIS == 0 ? SX : SY;
+  constexpr int EA = AXIS == 0 ? AXS : AYS;
+  const int b = (py + 2) * SY + px + 2;
+  const int ba = (py + 1) * AYS + px + 1;
   const int32_t v0 = s_phi[b], v1 = s_phi[b + E];
 
   // diffusion D B_a (phi(p) - phi(p + e)) with exact integer differences
   float dif;
-  if (DIM == 3 && AXIS == 0) {
-    // B_x = s_y s_z / 36
-    float acc = 0.f;
-#pragma unroll
-    for (int dz = -1; dz <= 1; dz++)
-#pragma unroll
-      for (int dy = -1; dy <= 1; dy++) {
-        const float wgt = (dy ? 1.f : 4.f) * (dz ? 1.f : 4.f);
-        const int o = dy * SY + dz * SZ;
-        acc = __fmaf_rn(wgt, dphi_of(s_phi[b + o], s_phi[b + o + E]), acc);
-      }
-    dif = __fmul_rn(acc, 1.0f / 36.0f);
-  } else if ((DIM == 3 && AXIS == 1) || (DIM == 2 && AXIS == 0)) {
-    // B = s_z / 6 (3D, y faces) or s_y / 6 (2D, x faces)
-    constexpr int T = DIM == 3 ? SZ : SY;
+  if (AXIS == 0) {
+    // B = s_y / 6
     float acc = __fmul_rn(4.f, dphi_of(v0, v1));
-    acc = __fadd_rn(acc, dphi_of(s_phi[b - T], s_phi[b - T + E]));
-    acc = __fadd_rn(acc, dphi_of(s_phi[b + T], s_phi[b + T + E]));
+    acc = __fadd_rn(acc, dphi_of(s_phi[b - SY], s_phi[b - SY + E]));
+    acc = __fadd_rn(acc, dphi_of(s_phi[b + SY], s_phi[b + SY + E]));
     dif = __fmul_rn(acc, 1.0f / 6.0f);
   } else {
     dif = dphi_of(v0, v1);
   }
   float tau = __fmul_rn(P.Dlap * (1.0f / 6.0f), dif);  // Dlap = 6 D
 
-  // compressive transfer 3 kappa W_a (a_a(p) + a_a(p + e)), W_a = s_b s_c / 216 (2D: s_b / 36)
+  // compressive transfer 3 kappa W_a (a_a(p) + a_a(p + e)), W_a = s_b / 36
   {
     const float *sa = s_a + AXIS * G::NA;
-    float acc = 0.f;
-    if (DIM == 3) {
-      constexpr int T1 = AXIS == 0 ? AYS : AXS, T2 = AXIS == 2 ? AYS : AZS;
-#pragma unroll
-      for (int d2 = -1; d2 <= 1; d2++)
-#pragma unroll
-        for (int d1 = -1; d1 <= 1; d1++) {
-          const float wgt = (d1 ? 1.f : 4.f) * (d2 ? 1.f : 4.f);
-          const int o = d1 * T1 + d2 * T2;
-          acc = __fmaf_rn(wgt, __fadd_rn(sa[ba + o], sa[ba + o + EA]), acc);
-        }
-      acc = __fmul_rn(acc, 1.0f / 216.0f);
-    } else {
-      constexpr int T1 = AXIS == 0 ? AYS : AXS;
-      acc = __fmul_rn(4.f, __fadd_rn(sa[ba], sa[ba + EA]));
-      acc = __fadd_rn(acc, __fadd_rn(sa[ba - T1], sa[ba - T1 + EA]));
-      acc = __fadd_rn(acc, __fadd_rn(sa[ba + T1], sa[ba + T1 + EA]));
-      acc = __fmul_rn(acc, 1.0f / 36.0f);
-    }
+    constexpr int T1 = AXIS == 0 ? AYS : AXS;
+    float acc = __fmul_rn(4.f, __fadd_rn(sa[ba], sa[ba + EA]));
+    acc = __fadd_rn(acc, __fadd_rn(sa[ba - T1], sa[ba - T1 + EA]));
+    acc = __fadd_rn(acc, __fadd_rn(sa[ba + T1], sa[ba + T1 + EA]));
+    acc = __fmul_rn(acc, 1.0f / 36.0f);
     tau = __fadd_rn(tau, __fmul_rn(P.kc * kCs2 * 3.0f, acc));  // kc = kappa / cs^2 -> 3 kappa
   }
 
@@ -112,14 +89,12 @@ __device__ __forceinline__ int32_t face_transfer(const KParams &P, const int32_t
     const int32_t s0 = minmod_i(v0 - vm, v1 - v0);
     const int32_t s1 = minmod_i(v1 - v0, vp - v1);
     // global cells p and p + e (periodic)
-    const int n0x = P.nx, n0y = P.ny, n0z = P.nz;
-    int qx = gx, qy = gy, qz = gz;
-    if (AXIS == 0) qx = qx == n0x - 1 ? 0 : qx + 1;
-    if (AXIS == 1) qy = qy == n0y - 1 ? 0 : qy + 1;
-    if (AXIS == 2) qz = qz == n0z - 1 ? 0 : qz + 1;
+    int qx = gx, qy = gy;
+    if (AXIS == 0) qx = qx == P.nx - 1 ? 0 : qx + 1;
+    if (AXIS == 1) qy = qy == P.ny - 1 ? 0 : qy + 1;
     const long long N = P.N;
-    const float ua = __ldg(u + AXIS * N + gx + (long long)n0x * (gy + (long long)n0y * gz));
-    const float ub = __ldg(u + AXIS * N + qx + (long long)n0x * (qy + (long long)n0y * qz));
+    const float ua = __ldg(u + AXIS * N + gx + (long long)P.nx * gy);
+    const float ub = __ldg(u + AXIS * N + qx + (long long)P.nx * qy);
     const float uf = __fmul_rn(0.5f, __fadd_rn(ua, ub));
     // upwind state; exact integer slopes, FP32 sum (no 64-bit conversion, which runs on the FP64 pipe)
     const float pup = uf >= 0.0f ? (__int2float_rn(v0) + 0.5f * __int2float_rn(s0)) * kInvQ30
@@ -129,33 +104,28 @@ __device__ __forceinline__ int32_t face_transfer(const KParams &P, const int32_t
   return __float2int_rn(__fmul_rn(tau, kQ30));
 }
 
-template <int DIM>
-__global__ void __launch_bounds__(PhaseGeom<DIM>::NT)
-k_phase(const KParams P, const int32_t *__restrict__ phi, const float *__restrict__ u,
-        int32_t *__restrict__ phi_out, const TileList next) {
+__global__ void __launch_bounds__(Phase2::NT)
+k_phase2(const KParams P, const int32_t *__restrict__ phi, const float *__restrict__ u,
+         int32_t *__restrict__ phi_out, const TileList next) {
   pdl_enter();
-  using G = PhaseGeom<DIM>;
-  using SL = typename StencilOf<DIM>::type;
+  using G = Phase2;
+  using SL = StencilOf<2>::type;
   __shared__ int32_t s_phi[G::NB];
-  __shared__ float s_a[3 * G::NA];
-  __shared__ int32_t s_tx[G::FX], s_ty[G::FY], s_tz[DIM == 3 ? G::FZ : 1];
+  __shared__ float s_a[2 * G::NA];
+  __shared__ int32_t s_tx[G::FX], s_ty[G::FY];
 
-  const int tx = threadIdx.x, ty = threadIdx.y, tz = threadIdx.z;
-  const int tid = tx + G::TX * (ty + G::TY * tz);
-  const int x0 = blockIdx.x * G::TX, y0 = blockIdx.y * G::TY, z0 = blockIdx.z * G::TZ;
-  const int nx = P.nx, ny = P.ny, nz = P.nz;
+  const int tx = threadIdx.x, ty = threadIdx.y;
+  const int tid = tx + G::TX * ty;
+  const int x0 = blockIdx.x * G::TX, y0 = blockIdx.y * G::TY;
+  const int nx = P.nx, ny = P.ny;
 
   // stage phi (halo 2) row by row: rows of HX = TX + 4 values
   int32_t some = 0;
   {
     const int xl = wrapn(x0 - 2 + tx, nx);
     const int xr = wrapn(x0 + 30 + (tx & 3), nx);
-    constexpr int NROWS = G::HY * G::HZ, NW = G::TY * G::TZ;
-    for (int r = ty + G::TY * tz; r < NROWS; r += NW) {
-      const int ry = r % G::HY, rz = r / G::HY;
-      const int Y = wrapn(y0 + ry - 2, ny);
-      const int Z = DIM == 3 ? wrapn(z0 + rz - 2, nz) : 0;
-      const int32_t *row = phi + (long long)nx * (Y + (long long)ny * Z);
+    for (int r = ty; r < G::HY; r += G::TY) {
+      const int32_t *row = phi + (long long)nx * wrapn(y0 + r - 2, ny);
       some |= s_phi[r * G::HX + tx] = row[xl];
       if (tx < 4) some |= s_phi[r * G::HX + 32 + tx] = row[xr];
     }
@@ -169,85 +139,65 @@ k_phase(const KParams P, const int32_t *__restrict__ phi, const float *__restric
   if (!__syncthreads_or(some)) {
     const int x = x0 + tx, y = y0 + ty;
     if (x < nx && y < ny) phi_out[(long long)x + (long long)nx * y] = 0;
-    if (next.tiles && tid == 0) next.mark[blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)] = 0;
+    if (next.tiles && tid == 0) next.mark[blockIdx.x + gridDim.x * blockIdx.y] = 0;
     return;
   }
 
   // compressive vector a = phi (1 - phi) grad(phi) / (|grad(phi)| + eps_n) on the tile + 1 halo
   for (int t = tid; t < G::NA; t += G::NT) {
-    const int ax = t % G::AX, ay = (t / G::AX) % G::AY, az = t / (G::AX * G::AY);
-    const int b = (DIM == 3 ? (az + 1) * G::HX * G::HY : 0) + (ay + 1) * G::HX + ax + 1;
-    float g0 = 0.f, g1 = 0.f, g2 = 0.f;
+    const int b = (t / G::AX + 1) * G::HX + t % G::AX + 1;
+    float g0 = 0.f, g1 = 0.f;
 #pragma unroll
     for (int i = 1; i < SL::Q; i++) {
       if (!positive<SL>(i)) continue;
-      const int o = SL::c(i, 0) + G::HX * (SL::c(i, 1) + G::HY * SL::c(i, 2));
+      const int o = SL::c(i, 0) + G::HX * SL::c(i, 1);
       const float d = SL::w(i) * dphi_of(s_phi[b + o], s_phi[b - o]);
       g0 += SL::c(i, 0) * d;
       g1 += SL::c(i, 1) * d;
-      if (DIM == 3) g2 += SL::c(i, 2) * d;
     }
-    g0 *= 3.0f; g1 *= 3.0f; g2 *= 3.0f;
+    g0 *= 3.0f; g1 *= 3.0f;
     const float ph = phi_of(s_phi[b]);
-    const float s = ph * (1.0f - ph) / (sqrtf(g0 * g0 + g1 * g1 + g2 * g2) + P.eps_n);
+    const float s = ph * (1.0f - ph) / (sqrtf(g0 * g0 + g1 * g1) + P.eps_n);
     s_a[t] = g0 * s;
     s_a[G::NA + t] = g1 * s;
-    s_a[2 * G::NA + t] = g2 * s;
   }
   __syncthreads();
 
-  // face transfers: x faces (TX + 1) x TY x TZ with the low face of the tile first
+  // face transfers: x faces (TX + 1) x TY with the low face of the tile first
   for (int t = tid; t < G::FX; t += G::NT) {
-    const int fx = t % (G::TX + 1), fy = (t / (G::TX + 1)) % G::TY, fz = t / ((G::TX + 1) * G::TY);
-    const int px = fx - 1;  // left cell, tile-local
-    const int gx = wrapn(x0 + px, nx), gy = wrapn(y0 + fy, ny), gz = DIM == 3 ? wrapn(z0 + fz, nz) : 0;
-    s_tx[t] = face_transfer<DIM, 0>(P, s_phi, s_a, u, px, fy, fz, gx, gy, gz);
+    const int px = t % (G::TX + 1) - 1, fy = t / (G::TX + 1);  // px: left cell, tile-local
+    s_tx[t] = face_transfer<0>(P, s_phi, s_a, u, px, fy, wrapn(x0 + px, nx), wrapn(y0 + fy, ny));
   }
   for (int t = tid; t < G::FY; t += G::NT) {
-    const int fx = t % G::TX, fy = (t / G::TX) % (G::TY + 1), fz = t / (G::TX * (G::TY + 1));
-    const int py = fy - 1;
-    const int gx = wrapn(x0 + fx, nx), gy = wrapn(y0 + py, ny), gz = DIM == 3 ? wrapn(z0 + fz, nz) : 0;
-    s_ty[t] = face_transfer<DIM, 1>(P, s_phi, s_a, u, fx, py, fz, gx, gy, gz);
-  }
-  if (DIM == 3) {
-    for (int t = tid; t < G::FZ; t += G::NT) {
-      const int fx = t % G::TX, fy = (t / G::TX) % G::TY, fz = t / (G::TX * G::TY);
-      const int pz = fz - 1;
-      const int gx = wrapn(x0 + fx, nx), gy = wrapn(y0 + fy, ny), gz = wrapn(z0 + pz, nz);
-      s_tz[t] = face_transfer<DIM, 2>(P, s_phi, s_a, u, fx, fy, pz, gx, gy, gz);
-    }
+    const int fx = t % G::TX, py = t / G::TX - 1;
+    s_ty[t] = face_transfer<1>(P, s_phi, s_a, u, fx, py, wrapn(x0 + fx, nx), wrapn(y0 + py, ny));
   }
   __syncthreads();
 
-  const int x = x0 + tx, y = y0 + ty, z = z0 + tz;
-  const bool inb = x < nx && y < ny && z < nz;
+  const int x = x0 + tx, y = y0 + ty;
   bool gated = false;
-  if (inb) {
-    const int b = (DIM == 3 ? (tz + 2) * G::HX * G::HY : 0) + (ty + 2) * G::HX + tx + 2;
-    int32_t acc = s_tx[tx + (G::TX + 1) * (ty + G::TY * tz)] - s_tx[tx + 1 + (G::TX + 1) * (ty + G::TY * tz)];
-    acc += s_ty[tx + G::TX * (ty + (G::TY + 1) * tz)] - s_ty[tx + G::TX * (ty + 1 + (G::TY + 1) * tz)];
-    if (DIM == 3) acc += s_tz[tx + G::TX * (ty + G::TY * tz)] - s_tz[tx + G::TX * (ty + G::TY * (tz + 1))];
-    const int32_t vn = s_phi[b] + acc;
-    phi_out[(long long)x + (long long)nx * (y + (long long)ny * z)] = vn;
+  if (x < nx && y < ny) {
+    int32_t acc = s_tx[tx + (G::TX + 1) * ty] - s_tx[tx + 1 + (G::TX + 1) * ty];
+    acc += s_ty[tx + G::TX * ty] - s_ty[tx + G::TX * (ty + 1)];
+    const int32_t vn = s_phi[(ty + 2) * G::HX + tx + 2] + acc;
+    phi_out[(long long)x + (long long)nx * y] = vn;
     gated = q_gate_value(vn) >= P.q_th;
   }
   if (next.tiles) {  // one block per tile: it sets the tile's mark either way
     const int any = __syncthreads_or(gated);
     if (tid == 0) {
-      const int tile = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
+      const int tile = blockIdx.x + gridDim.x * blockIdx.y;
       next.mark[tile] = any != 0;
       if (any) next.tiles[atomicAdd(next.count, 1)] = tile;
     }
   }
 }
 
-template <int DIM>
-static cudaError_t launch_phase_dim(const KParams &P, const int32_t *phi, const float *u, int32_t *phi_out,
-                                    const TileList &next, cudaStream_t s) {
-  using G = PhaseGeom<DIM>;
-  dim3 block(G::TX, G::TY, G::TZ);
-  dim3 grid((P.nx + G::TX - 1) / G::TX, (P.ny + G::TY - 1) / G::TY, (P.nz + G::TZ - 1) / G::TZ);
-  return launch_pdl(k_phase<DIM>, grid, block, 0, s, P, phi, u, phi_out, next);
+static cudaError_t launch_phase2(const KParams &P, const int32_t *phi, const float *u, int32_t *phi_out,
+                                 const TileList &next, cudaStream_t s) {
+  using G = Phase2;
+  dim3 grid((P.nx + G::TX - 1) / G::TX, (P.ny + G::TY - 1) / G::TY);
+  return launch_pdl(k_phase2, grid, dim3(G::TX, G::TY), 0, s, P, phi, u, phi_out, next);
 }
 
 // Records once, at context creation, how many k_phase3m blocks the device holds at once (SMs x
@@ -302,7 +252,7 @@ static cudaError_t launch_phase3(const KParams &P, const int32_t *phi, const flo
 
 cudaError_t launch_phase(int dim, const KParams &P, const int32_t *phi, const float *u, int32_t *phi_out,
                          const TileList &next, const TileList &prev, cudaStream_t s) {
-  return dim == 2 ? launch_phase_dim<2>(P, phi, u, phi_out, next, s)
+  return dim == 2 ? launch_phase2(P, phi, u, phi_out, next, s)
                   : launch_phase3(P, phi, u, phi_out, next, prev, s);
 }
 
