@@ -12,6 +12,10 @@ namespace lbm {
 // The case record of the next item is copied into shared memory (double-buffered) while the
 // current item computes, so an item starts without a chain of dependent global loads, and its
 // parameters are read from shared memory.
+// Blocks per SM: the item loop holds more than the single-case kernel does, so the bounds are its own.
+// The pass over 24 cubes of 48 to 96 cells, the fastest tile shape of each: D3Q19 six in FP32 368 us (80
+// registers, 32 bytes spilt; five, without a spill, 371) and six in FP16 332 (44 spilt; seven 352, five
+// 354); D3Q27 four 507 and in FP16 460 us, where five take 488 and 425.
 template <class L, int S, int TY>
 __global__ void __launch_bounds__(LX * 8, L::Q >= 27 ? 4 : 6)
 k_hydro2_batch(const BatchCase *__restrict__ cases, const int4 *__restrict__ items, const int nitems) {
@@ -116,7 +120,7 @@ cudaError_t launch_hydro_batch(int Q, int store, int ty, const BatchCase *cases,
 }
 
 int hydro_batch_blocks(int Q, int store, int ty) {
-  // the resident count depends on the lattice (registers), not on the store or the tile shape
+  // the resident count depends on the lattice (the launch bounds), not on the store or the tile shape
   (void)store; (void)ty;
   return Q == 27 ? resident(k_hydro2_batch<D3Q27, 0, 4>, LX * 8) : resident(k_hydro2_batch<D3Q19, 0, 4>, LX * 8);
 }

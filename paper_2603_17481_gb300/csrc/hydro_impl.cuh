@@ -691,8 +691,9 @@ __device__ __forceinline__ void hydro2_prefetch(const KParams &P, const typename
 
 // Tile of the paired kernel in y and z, and the blocks per SM its registers are sized for: D3Q19 six
 // in FP32 (80 registers: 128.2 us on 256 x 128 x 128; seven at 72 spill: 135.0, five 148.5) and seven
-// with 2-byte stores (107.9; six 109.5, eight 120.9), D3Q27 five (96 registers: 64.2 us on
-// 160 x 96 x 96; six 71.7, four 69.6).
+// with 2-byte stores (72 registers: 107.9, although the step spills 88 bytes; six 109.5, eight 120.9),
+// D3Q27 five (96 registers: 64.2 us in FP32 on 160 x 96 x 96; six 71.7, four 69.6; with 2-byte stores
+// the step spills 52 bytes).
 struct HydroTile {
   static constexpr int Y = 2, Z = 4;
 };
@@ -704,14 +705,18 @@ static_assert(NciTile<3>::X == 2 * LX && NciTile<3>::Y == 4 * HydroTile::Y && Nc
 __device__ __forceinline__ int nci_tile_of(const KParams &P, int bx, int by, int bz) {
   return bx + ((P.nx + 31) >> 5) * ((by >> 2) + ((P.ny + 7) >> 3) * bz);
 }
-// The blocks that ask L2 for their rows: about the first resident wave of a 152-SM GB300.
+// The blocks that ask L2 for their rows: the first resident wave of a 152-SM GB300 at six blocks per SM, one
+// number for all kernels (D3Q27 has five, 2-byte D3Q19 seven).
 constexpr unsigned kPrefetchBlocks = 912;
 
 // listed == nullptr: every cell. Otherwise the split step's first part: only the tiles whose
 // near-contact tile is not listed.
 // The first blocks of the grid, which may be resident while the previous kernel still runs, ask L2
-// for their population rows before they wait for it (128.5 -> 127.0 us on 256 x 128 x 128; asked by
-// every block it cost 384^3 6 %: 1785 us against 1682; both with tiles of 64 x 2 x 2 cells).
+// for their population rows before they wait for it. With tiles of 64 x 2 x 2 cells that took 128.5 to
+// 127.0 us on 256 x 128 x 128 (asked by every block it cost 384^3 6 %: 1785 us against 1682). With the
+// present tiles it is worth little either way: a step with it and without, D3Q19 96^3 63.0 / 63.3 us,
+// 256 x 128 x 128 207.2 / 206.2 and in FP16 187.3 / 185.3, D3Q27 160 x 96 x 96 102.4 / 103.0, 256 x 128 x 128
+// 250.6 / 249.6 and in FP16 220.8 / 217.3; lbm_mass with the moments pass 214.6 / 211.3 (D3Q19), 245.2 / 247.0.
 template <class L, int S, int MODE>
 __global__ void __launch_bounds__(kHydro2Threads, hydro2_minb<L, S>())
 k_hydro2(const KParams P, const typename Store<S>::T *__restrict__ src, typename Store<S>::T *__restrict__ dst,

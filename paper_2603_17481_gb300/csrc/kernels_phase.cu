@@ -131,11 +131,14 @@ k_phase2(const KParams P, const int32_t *__restrict__ phi, const float *__restri
     }
   }
   // Where phi is exactly zero in the tile and its halo (gas further from every interface than the
-  // profiles reach), each transfer of the tile is zero, since phi, its differences and the compressive
-  // vector are: phi stays zero and holds no interfacial cell. 1021 x 509 with two droplets of radius 96,
-  // 200 steps: 29.3 -> 24.9 us a step. (The diffusive tails grow as 3 sqrt(t) cells until they round to zero,
-  // so the 3D grids, at most 128 cells across, are full after 50 steps: there the same test gained 9 % of the
-  // march on 256 x 128 x 128 and cost a third of it on 160 x 96 x 96, and was not kept.)
+  // profiles and their diffusive tails reach), each transfer of the tile is zero, since phi, its
+  // differences and the compressive vector are: phi stays zero and holds no interfacial cell. The tails
+  // grow as 3 sqrt(t) cells at first and slow down as they round to zero, so the gain lasts but shrinks.
+  // A step of 1021 x 509 with two droplets of radius 96, with the test and without it: at step 100 27.1
+  // and 31.1 us (773 of 1024 tiles empty), at 4000 28.0 and 31.2 (559), at 16000 29.0 and 30.8 (355); on
+  // 2048 x 2048 106.5 and 162.5, at step 16000 110 and 162.
+  // (In the 3D march the same test did not pay: it gained 9 % of the pass on 256 x 128 x 128 and cost a third of
+  // it on 160 x 96 x 96, and both grids are full after about 50 steps.)
   if (!__syncthreads_or(some)) {
     const int x = x0 + tx, y = y0 + ty;
     if (x < nx && y < ny) phi_out[(long long)x + (long long)nx * y] = 0;
